@@ -976,9 +976,18 @@ __global__ void __launch_bounds__(kThreads) k_pack_local(const T* __restrict__ s
     return;
   }
   // b_spec < 0: the statistics are already in the header (an epilogue merged
-  // them): the width is exact and every tile goes straight to its place
+  // them): the width is exact and every tile goes straight to its place,
+  // unless it is past -b_spec, the widest that the capacity holds (k_repack
+  // then reports that)
   const bool exact = b_spec < 0;
-  if (exact) b_spec = width_from_stats(out->stat_or, out->stat_neg);
+  if (exact) {
+    const int widest = -b_spec;
+    b_spec = width_from_stats(out->stat_or, out->stat_neg);
+    if (b_spec > widest) {
+      cp_async_wait0_ge();
+      return;
+    }
+  }
   uint64_t g_or = 0;
   uint32_t g_neg = 0;
   int cur = 0;

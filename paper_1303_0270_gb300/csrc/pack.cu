@@ -487,7 +487,7 @@ void run_pack_scratch32(const int32_t* vals, const ccm_matrix& out, cudaStream_t
   const int cls = ew_class(width_bound(out.capacity, n));
   if (cls && n && reinterpret_cast<uintptr_t>(vals) % 16 == 0) {
     // the producer merged the statistics: one pass at the exact width (the
-    // staged single-pass kernel, spec < 0), then the header
+    // staged single-pass kernel, spec < 0: minus the widest width), then the header
     ge::EwCall c{};
     c.kind = ge::EwKind::LocalI32;
     c.dense = vals;
@@ -497,7 +497,7 @@ void run_pack_scratch32(const int32_t* vals, const ccm_matrix& out, cudaStream_t
     c.rows = out.rows;
     c.cols = out.cols;
     c.slot_class = cls;
-    c.spec = -1;
+    c.spec = -width_bound(out.capacity, n);
     launch_ew(cls, c, st);
     c.kind = ge::EwKind::Repack;
     launch_ew(cls, c, st);
