@@ -121,7 +121,8 @@ typedef enum ccm_op {
 /* Matmul paths. */
 typedef enum ccm_matmul_path {
   CCM_MATMUL_AUTO = 0,
-  CCM_MATMUL_TENSOR = 1,  /* exact 4-bit limb decomposition on the tcgen05 tensor cores */
+  CCM_MATMUL_TENSOR = 1,  /* exact digit decomposition on the tcgen05 tensor cores (operands
+                             of at most 16 bits; AUTO takes it for wider ones too) */
   CCM_MATMUL_CUDACORE = 2 /* decode-and-multiply on the integer ALUs */
 } ccm_matmul_path;
 
@@ -237,7 +238,8 @@ ccm_status ccm_matmul(const ccm_matrix* a, const ccm_matrix* b, const ccm_matrix
 
 /* Device workspace needed by `op` on an m x k by k x n problem (matvec: n = 1
  * is the vector, k the inner size).  An upper bound over all operand widths
- * (for matmul: the tensor path's digit planes at 4 digits per field).  For
+ * (for matmul: the tensor path's digit planes, three 2-byte digits per field;
+ * with less, a product that would need more runs on the CUDA cores).  For
  * CCM_OP_PACK the arguments are (rows, cols, output capacity in words). */
 size_t ccm_workspace_bytes(int op, uint64_t m, uint64_t k, uint64_t n);
 

@@ -180,7 +180,7 @@ ccm_status ccm_matmul(const ccm_matrix* a, const ccm_matrix* b, const ccm_matrix
   if (b->rows != a->cols || c->rows != a->rows || c->cols != b->cols) return CCM_E_SHAPE;
   if (!capacity_ok(c)) return CCM_E_CAPACITY;
   if (ws_bytes < ccm::matmul_workspace(*a, *b)) return CCM_E_CAPACITY;  // <= the shape bound
-  int st = ccm::run_matmul(*a, *b, *c, path, ws, to_cuda(stream));
+  int st = ccm::run_matmul(*a, *b, *c, path, ws, ws_bytes, to_cuda(stream));
   if (st != CCM_OK) return (ccm_status)st;
   return launched();
 }

@@ -10,8 +10,10 @@
 namespace ccm {
 namespace ax {
 
-// Polls of one bounded wait before it gives up; with the globaltimer check
-// below a wait never lasts more than about two seconds.
+// A bounded wait suspends for up to kSuspendNs at a time (the hint of
+// try_wait; without it a waiting warp polls and its polls hold up the shared
+// memory accesses of the others), and gives up after about two seconds.
+constexpr uint32_t kSuspendNs = 1000000;
 constexpr uint32_t kSpinLimit = 1u << 26;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -40,7 +42,8 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 }
 
 // Bounded wait for the phase of parity `parity` to complete: false after
-// about two seconds (or kSpinLimit polls), never an endless spin.
+// about two seconds (or kSpinLimit polls), never an endless spin.  The clock
+// is read only after a failed poll.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   const uint32_t addr = smem_u32(bar);
   uint64_t t0 = 0;
@@ -48,19 +51,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
         "selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(addr), "r"(parity)
+        : "r"(addr), "r"(parity), "r"(kSuspendNs)
         : "memory");
     if (done) return true;
-    if ((it & 1023) == 0) {
-      const uint64_t now = globaltimer_ns();
-      if (it == 0)
-        t0 = now;
-      else if (now - t0 > 2000000000ull)
-        return false;
-    }
+    const uint64_t now = globaltimer_ns();
+    if (it == 0)
+      t0 = now;
+    else if (now - t0 > 2000000000ull)
+      return false;
   }
   return false;
 }

@@ -68,12 +68,14 @@ void run_matvec(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, v
 void run_repack(const ccm_matrix& in, int width, int is_signed, const ccm_matrix& out,
                 uint64_t row_offset, cudaStream_t st);
 
+// The least workspace ccm_matmul accepts.
 size_t matmul_workspace(const ccm_matrix& a, const ccm_matrix& b);
-// Shape-only bound on matmul_workspace (the widths are unknown): the tensor
-// path at its widest (4 digits per field).
+// What ccm_workspace_bytes gives for a shape (the widths are unknown): enough
+// for the tensor path at its widest.  With less (but at least
+// matmul_workspace) a product may run on the CUDA cores instead.
 size_t matmul_workspace_upper(uint64_t m, uint64_t k, uint64_t n);
 int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, int path, void* ws,
-               cudaStream_t st);
+               size_t ws_bytes, cudaStream_t st);
 
 size_t vlb_workspace(uint64_t n);
 size_t vlb_matvec_workspace(uint64_t rows);

@@ -165,23 +165,58 @@ __global__ void __launch_bounds__(256) k_matmul_cc32(ccm_header* out, const ccm_
 
 }  // namespace
 
+namespace {
+
+size_t c_scratch_bytes(uint64_t m, uint64_t n) {
+  return ((m * n * sizeof(int64_t)) + 255) & ~(size_t)255;
+}
+
+// Digits of 4 bits of the wider operand (by the capacities) when the explicit
+// tensor path (CCM_MATMUL_TENSOR) takes the product: at most 4, with every
+// sum of 4-bit digit products below 2^24; else 0.
+int nibble_digits(const ccm_matrix& a, const ccm_matrix& b) {
+  const uint64_t m = a.rows, k = a.cols, n = b.cols;
+  if (!m || !n || !k) return 0;
+  const int ba = width_bound(a.capacity, m * k), bb = width_bound(b.capacity, k * n);
+  const int L = (max(ba, bb) + 3) / 4;
+  if (L < 1 || L > 4) return 0;
+  if ((double)k * L * 225.0 >= 16777216.0) return 0;
+  return ba + bb + bitlen_host(k) <= 62 ? L : 0;
+}
+
+}  // namespace
+
+// One byte per field and 4-bit digit, both operands padded to whole tiles.
+static size_t nibble_bytes(uint64_t m, uint64_t k, uint64_t n, int L) {
+  auto up = [](uint64_t v, uint64_t to) { return (v + to - 1) / to * to; };
+  const uint64_t kp = up(k, 128), np = up(n, L == 1 ? 256 : L == 2 ? 128 : 64);
+  return up(L * up(m, 128) * kp, 256) + up(L * np * kp, 256);
+}
+
+// The least workspace ccm_matmul accepts: C in int64, plus one byte per field
+// and 4-bit digit where the explicit tensor path applies.
 size_t matmul_workspace(const ccm_matrix& a, const ccm_matrix& b) {
-  const uint64_t m = a.rows, n = b.cols;
-  size_t c_bytes = ((m * n * sizeof(int64_t)) + 255) & ~(size_t)255;
-  return c_bytes + matmul_tc_workspace(a, b) + 256;
+  const int L = nibble_digits(a, b);
+  return c_scratch_bytes(a.rows, b.cols) + 256 +
+         (L ? nibble_bytes(a.rows, a.cols, b.cols, L) : 0);
 }
 
 size_t matmul_workspace_upper(uint64_t m, uint64_t k, uint64_t n) {
-  size_t c_bytes = ((m * n * sizeof(int64_t)) + 255) & ~(size_t)255;
-  return c_bytes + matmul_tc_workspace_upper(m, k, n) + 256;
+  const size_t digits = m && n && k ? umax(matmul_tc_bytes_upper(m, k, n),
+                                           nibble_bytes(m, k, n, 4)) : 0;
+  return c_scratch_bytes(m, n) + digits + 256;
 }
 
 int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, int path, void* ws,
-               cudaStream_t st) {
+               size_t ws_bytes, cudaStream_t st) {
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  const bool tc_ok = matmul_tc_supported(a, b);
-  if (path == CCM_MATMUL_TENSOR && !tc_ok) return CCM_E_SHAPE;
-  const bool tc = tc_ok && (path == CCM_MATMUL_TENSOR || path == CCM_MATMUL_AUTO);
+  if (path == CCM_MATMUL_TENSOR && (!nibble_digits(a, b) || !matmul_tc_applies(a, b)))
+    return CCM_E_SHAPE;
+  bool tc = path != CCM_MATMUL_CUDACORE && matmul_tc_applies(a, b);
+  if (tc && ws_bytes < c_scratch_bytes(m, n) + matmul_tc_bytes(a, b)) {
+    if (path == CCM_MATMUL_TENSOR) return CCM_E_CAPACITY;
+    tc = false;
+  }
   int64_t* cs = (int64_t*)ws;
   InitArgs ia{};
   ia.out = c.hdr;
@@ -202,8 +237,7 @@ int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, in
   launch_init(ia, st);
   if (m && n && k) {
     if (tc) {
-      size_t c_bytes = ((m * n * sizeof(int64_t)) + 255) & ~(size_t)255;
-      int rc = run_matmul_tc(a, b, c, cs, (char*)ws + c_bytes, st);
+      int rc = run_matmul_tc(a, b, c, cs, (char*)ws + c_scratch_bytes(m, n), st);
       if (rc != CCM_OK) return rc;
       if (matmul_c32(c))
         run_pack_scratch32(reinterpret_cast<const int32_t*>(cs), c, st);

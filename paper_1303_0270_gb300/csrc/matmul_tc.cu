@@ -1,39 +1,50 @@
 // matmul_tc.cu -- exact integer C = A B on the tcgen05 tensor cores.
 //
 // GB300 (sm_103a) has no integer tensor-core MMA (tcgen05.mma .kind::i8 is
-// rejected by ptxas for this target), so the product is computed through an
-// exact decomposition into 4-bit digits, which e4m3 represents exactly:
+// rejected by ptxas for this target), so the product runs on fp16 operands
+// whose values are integers, accumulated in fp32:
 //
-//   a = sum_{l < L} d_l 16^l,  d_l in [0, 15] for l < L-1,  d_{L-1} = a >> 4(L-1)
+//   a = sum_l d_l 2^(w l),   l = 0 .. d-1,   |d_l| <= 2^(w-1)   (balanced digits)
+//   C = sum_{l, m} 2^(w_a l + w_b m) (A_l B_m)
 //
-// (two's complement bits for the low digits, an arithmetic shift for the top
-// one, so the top digit is in [-8, 7] for signed fields and [0, 15] for
-// unsigned ones; L = ceil(b / 4)).  Then
+// With e the width of a field as a two's complement number (b for signed
+// matrices, b + 1 for unsigned ones), d digits need w = ceil(e / d) bits.
+// fp16 holds every integer up to 2^11, so a digit may have up to 12 bits and
+// fields of up to 12 bits are one digit.  Products of magnitudes 2^p and 2^q
+// are integers; a sum of 2^(24 - p - q) of them is at most 2^24, so every
+// partial sum of such a run of k is an integer that fp32 holds exactly in
+// whatever order it is formed.  The product of every digit pair is therefore
+// accumulated in tensor memory over runs of k of at most that length (at
+// least kMinRun), and the epilogue warps add each run to integer accumulators
+// in registers while the next run is being multiplied.
 //
-//   C = sum_c 16^c S_c,   S_c = sum_{l + m = c} A_l B_m,
+// Why fp16 and not e4m3: fp8 runs at twice the rate but holds 4 significant
+// bits, so an 8 x 8-bit product takes 4 fp8 MMAs (2 units of fp16 time) where
+// one fp16 MMA does, a 12 x 12-bit one 9 (4.5 units) instead of 2, a
+// 16 x 16-bit one 16 (8 units) instead of 4.
 //
-// and every S_c is a dense e4m3 x e4m3 GEMM accumulated in fp32 in tensor
-// memory.  Each product of two digits is at most 225 in magnitude, so an
-// S_c entry is at most L * k * 225 < 2^24 whenever k * L * 225 < 2^24: every
-// partial sum is an integer that fp32 holds exactly, and the epilogue
-// converts S_c to int64 and combines the classes exactly.
+// Measured on GB300 (whole call; before: e4m3 digits in one-CTA tiles, or the
+// CUDA cores above 16 bits): 4096^3 at 4 / 8 / 12 / 16 signed bits 0.21 / 0.39 /
+// 0.92 / 1.31 -> 0.14 / 0.15 / 0.55 / 0.56 ms; 3001 x 2503 x 3500 at 20 x 18
+// bits 8.30 -> 0.37 ms.  What bounds it: the L2, which feeds the stages about
+// 46 bytes per clock and SM; above 32-bit sums also the conversions of short
+// runs (12 x 12 bits: runs of 256).
 //
-// Pipeline (one CTA of 4 warps per 128 x BN output tile):
-//   k_limbs_a / k_limbs_bt  packed A, B -> digit planes in e4m3, K-major,
-//                           zero padded to the tile sizes (B transposed)
-//   k_mm_tc                 warp 0: TMA producer (128-byte swizzled tiles of
-//                           every digit plane, mbarrier pipeline); warp 1:
-//                           one thread issues tcgen05.mma for every digit
-//                           pair into the accumulator of its class; all four
-//                           warps: epilogue (tcgen05.ld, exact int64 combine,
-//                           width statistics of C merged into C's header)
-// The int64 C is then packed by the pack pass of the pack engine.
+// Kernels:
+//   k_planes  packed A and B -> fp16 digit planes, K-major (B transposed)
+//   k_mm      persistent pairs of CTAs (one tcgen05 cta_group::2 tile of
+//             256 x BN outputs per pair): warp 0 TMA producer, warp 1 MMA
+//             issuer (leader CTA), warps 4-11 epilogue
 //
 // Every wait on an mbarrier is bounded; a wait that gives up records
-// CCM_E_TIMEOUT in C's header and the CTA frees its tensor memory and exits.
+// CCM_E_TIMEOUT in C's header and the CTAs free their tensor memory and exit.
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
+#include "async_copy.cuh"
 #include "ccm_device.cuh"
 #include "kernels.h"
 #include "matmul_tc.h"
@@ -41,302 +52,277 @@
 namespace ccm {
 namespace tc {
 
-constexpr int kBM = 128;    // rows of A / C per tile (UMMA M)
-constexpr int kBK = 128;    // K elements (= bytes of e4m3) per pipeline stage
-constexpr uint32_t kSpinLimit = 1u << 26;  // bounded mbarrier waits
-constexpr uint32_t kGroupM = 8;            // tile rows per raster group
+using ax::mbar_init;
+using ax::mbar_wait;
+using ax::smem_u32;
 
-// Tile geometry for L digits per operand.
-struct Geo {
-  int L = 0;        // digits per field
-  int classes = 0;  // 2L - 1 accumulators
-  int bn = 0;       // UMMA N
-  int stages = 0;
-  int accs = 0;     // accumulator sets in tensor memory (2: a tile's epilogue
-                    // overlaps the next tile's MMAs)
-  int tmem_cols = 0;
+constexpr int kBM = 256;          // rows of C per CTA pair (128 per CTA)
+constexpr int kBK = 64;           // fp16 elements of a block of k (a 128-byte swizzled row)
+constexpr uint32_t kGroupM = 4;   // tile rows per raster group
+constexpr int kMaxDigits = 3;
+constexpr int kMaxMag = 11;       // fp16 integers are exact up to 2^11
+constexpr int kMinRun = 256;      // shortest run of k between two flushes
+
+// Digit counts and widths of one product.
+struct Split {
+  uint8_t da, wa, db, wb;
+  // k elements whose products stay exact in fp32 (a multiple of kBK)
+  __host__ __device__ int run() const { return 1 << (26 - wa - wb); }
 };
 
-__host__ __device__ constexpr Geo geometry(int L) {
-  Geo g;
-  g.L = L;
-  g.classes = 2 * L - 1;
-  g.bn = L == 1 ? 256 : (L == 2 ? 128 : 64);
-  const int stage_bytes = L * kBK * (kBM + g.bn);
-  g.stages = 200 * 1024 / stage_bytes;
-  if (g.stages > 4) g.stages = 4;
-  const int cols = g.classes * g.bn;
-  g.accs = 2 * cols <= 512 ? 2 : 1;
-  int p = 32;
-  while (p < g.accs * cols) p <<= 1;
-  g.tmem_cols = p;
-  return g;
+// The cheapest split for operands of e_a and e_b bits (two's complement),
+// 1 .. kMaxE each: fewest digit pairs, then the longest run.  da = 0: none
+// fits.  A table, because every CTA asks for it once it knows the widths.
+constexpr int kMaxE = 32;
+struct SplitTable {
+  Split at[kMaxE + 1][kMaxE + 1];
+};
+constexpr SplitTable make_splits() {
+  SplitTable t{};
+  for (int ea = 1; ea <= kMaxE; ++ea)
+    for (int eb = 1; eb <= kMaxE; ++eb) {
+      int best = 1 << 30;
+      for (int da = 1; da <= kMaxDigits; ++da)
+        for (int db = 1; db <= kMaxDigits; ++db) {
+          const int wa = (ea + da - 1) / da, wb = (eb + db - 1) / db;
+          const int mags = wa + wb - 2;
+          if (wa - 1 > kMaxMag || wb - 1 > kMaxMag || mags > 16 ||
+              (kMinRun << mags) > (1 << 24))
+            continue;
+          const int score = da * db * 64 + mags;
+          if (score < best) {
+            best = score;
+            t.at[ea][eb].da = (uint8_t)da;
+            t.at[ea][eb].wa = (uint8_t)wa;
+            t.at[ea][eb].db = (uint8_t)db;
+            t.at[ea][eb].wb = (uint8_t)wb;
+          }
+        }
+    }
+  return t;
+}
+constexpr SplitTable kSplits = make_splits();
+__constant__ SplitTable c_splits = make_splits();
+
+// The split of the two headers' widths (the host has bounded both by 31).
+__device__ __forceinline__ Split split_of(const ccm_header* ha, const ccm_header* hb) {
+  const int ea = ha->width + !ha->is_signed, eb = hb->width + !hb->is_signed;
+  if (ea > kMaxE || eb > kMaxE) return Split{0, 0, 0, 0};
+  return c_splits.at[ea][eb];
 }
 
 __host__ __device__ inline uint64_t round_up(uint64_t v, uint64_t m) { return (v + m - 1) / m * m; }
 
 // ---------------------------------------------------------------------------
-// e4m3 encoding of a digit in [-8, 15] (exact: at most 4 significant bits).
+// Digit planes
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint8_t e4m3_of_digit(int d) {
-  if (d == 0) return 0;
-  uint32_t sign = d < 0 ? 0x80u : 0u;
-  uint32_t v = (uint32_t)(d < 0 ? -d : d);  // 1..15
-  int e = 31 - __clz(v);                    // 0..3
-  uint32_t mant = (v << (3 - e)) & 7u;
-  return (uint8_t)(sign | ((uint32_t)(e + 7) << 3) | mant);
-}
-
-__device__ __forceinline__ int digit(int64_t a, int l, int L) {
-  return l == L - 1 ? (int)(a >> (4 * l)) : (int)((a >> (4 * l)) & 15);
-}
-
-// ---------------------------------------------------------------------------
-// Fields of exactly 4L bits: digit l of field f is nibble f L + l of the
-// packed stream (the stream is LSB-first and the digits are the value's
-// nibbles, the top one taken as signed for two's complement fields), so the
-// digit planes are a strided nibble gather.  Four nibbles become four e4m3
-// bytes by table lookup with byte permutes: the low three bits of a nibble
-// select a byte of an 8-byte table (entries 0..7, or 8..15 / the negative
-// digits -8..-1), bit 3 picks which table.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t e4m3_of_nibbles(uint32_t x, bool top_signed) {
-  // e4m3 of 0..7, 8..15, and of -8..-1 (nibbles 8..15 of a signed digit)
-  constexpr uint32_t kLo0 = 0x44403800u, kLo1 = 0x4E4C4A48u;
-  constexpr uint32_t kHi0 = 0x53525150u, kHi1 = 0x57565554u;
-  constexpr uint32_t kNeg0 = 0xCACCCED0u, kNeg1 = 0xB8C0C4C8u;
-  const uint32_t sel = x & 0x7777u;
-  const uint32_t lo = __byte_perm(kLo0, kLo1, sel);
-  const uint32_t hi = top_signed ? __byte_perm(kNeg0, kNeg1, sel) : __byte_perm(kHi0, kHi1, sel);
-  const uint32_t big = __byte_perm(0u, 0xFFFFFFFFu, (x >> 1) & 0x4444u);  // 0xFF where bit 3
-  return (lo & ~big) | (hi & big);
-}
-
-// The 8 digit bytes of plane l for 8 consecutive fields held in w[0..L)
-// (32 L bits: 8 fields of 4L bits), as two words (fields 0..3, 4..7).
-template <int L>
-__device__ __forceinline__ uint2 plane_bytes8(const uint32_t (&w)[L], int l, bool top_signed) {
-  uint32_t x0 = 0, x1 = 0;
+// Eight consecutive fields of B bits of a packed stream from field e0 on
+// (`cnt` of them; the others read as zero): all their words loaded at once (no
+// word past the last field), moved to a common start, and cut with shifts
+// fixed at compile time.
+template <int B>
+__device__ __forceinline__ void decode8(const uint32_t* __restrict__ words, uint64_t e0, int cnt,
+                                        int sgn, int (&v)[8]) {
+  constexpr int kX = (8 * B + 31) / 32;  // aligned words
+  const uint64_t p = e0 * (uint64_t)B;
+  const uint32_t* q = words + (p >> 5);
+  const uint32_t s = (uint32_t)p & 31;
+  const int need = (int)(s + max(cnt, 0) * B + 31) >> 5;
+  uint32_t w[kX + 1], x[kX];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int j = q * L + l;  // nibble index in the 8-field group
-    const uint32_t nib = (w[j >> 3] >> (4 * (j & 7))) & 15u;
-    if (q < 4)
-      x0 |= nib << (4 * q);
+  for (int j = 0; j <= kX; ++j) w[j] = j < need && cnt > 0 ? __ldg(q + j) : 0u;
+#pragma unroll
+  for (int j = 0; j < kX; ++j) x[j] = __funnelshift_r(w[j], w[j + 1], s);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int bit = j * B, wi = bit >> 5, sh = bit & 31;
+    uint32_t t;  // the field at the top of the word
+    if (sh + B <= 32)
+      t = x[wi] << (32 - B - sh);
     else
-      x1 |= nib << (4 * (q - 4));
+      t = __funnelshift_r(x[wi], x[wi + 1 < kX ? wi + 1 : wi], sh) << (32 - B);
+    v[j] = sgn ? (int)t >> (32 - B) : (int)(t >> (32 - B));
   }
-  return make_uint2(e4m3_of_nibbles(x0, top_signed), e4m3_of_nibbles(x1, top_signed));
+  if (cnt < 8) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j >= cnt) v[j] = 0;
+  }
 }
 
-// The L words holding fields [f0, f0 + 8) of a stream of 4L-bit fields (f0 a
-// multiple of 8, so the group starts on a word).
-template <int L>
-__device__ __forceinline__ void load_group8(const uint32_t* __restrict__ w, uint64_t f0,
-                                            uint32_t (&out)[L]) {
-  const uint32_t* p = w + f0 * L / 8;
-  if constexpr (L == 1) {
-    out[0] = __ldg(p);
-  } else if constexpr (L == 2) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-    out[0] = v.x;
-    out[1] = v.y;
-  } else if constexpr (L == 4) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-    out[0] = v.x;
-    out[1] = v.y;
-    out[2] = v.z;
-    out[3] = v.w;
+// Splits off the low balanced digit of w bits: v becomes the rest.
+__device__ __forceinline__ int take_digit(int& v, int w) {
+  const int d = (int)((uint32_t)v << (32 - w)) >> (32 - w);
+  v = (v >> w) + ((v >> (w - 1)) & 1);
+  return d;
+}
+
+// Two integers as halves.  Magnitudes of at most 256 (`small`): 0x6600 is
+// 1536 = 1.5 * 2^10, whose ulp is 1, so adding the integer to its bits adds it
+// to its value, and the subtraction is exact (the conversion instruction runs
+// at a fraction of that rate).
+__device__ __forceinline__ uint32_t half2_bits(int x, int y, bool small) {
+  __half2 h;
+  if (small) {
+    const uint32_t u = (uint32_t)x + ((uint32_t)y << 16) + 0x66006600u, base = 0x66006600u;
+    h = __hsub2(*reinterpret_cast<const __half2*>(&u), *reinterpret_cast<const __half2*>(&base));
   } else {
-#pragma unroll
-    for (int i = 0; i < L; ++i) out[i] = __ldg(p + i);
+    h = __halves2half2(__int2half_rn(x), __int2half_rn(y));
   }
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// A (m x k, row-major, k % 8 == 0) with fields of exactly 4L bits ->
-// planes [L][m_pad][k_pad]: thread per 8 consecutive fields of a row.
-template <int L>
-__device__ void limbs_a_nibbles(const uint32_t* __restrict__ w, int sgn, uint64_t m, uint64_t k,
-                                uint64_t m_pad, uint64_t k_pad, uint8_t* __restrict__ planes) {
-  const uint64_t plane = m_pad * k_pad;
-  const uint32_t groups = (uint32_t)(k_pad / 8);
-  for (uint64_t i = blockIdx.x; i < m_pad; i += gridDim.x) {
-    for (uint32_t q = threadIdx.x; q < groups; q += blockDim.x) {
-      const uint64_t kk = 8ull * q;
-      uint2 out[L];
-      if (i < m && kk < k) {
-        uint32_t wg[L];
-        load_group8<L>(w, i * k + kk, wg);
+struct PlaneArgs {
+  const ccm_header *out, *ha, *hb;
+  const uint32_t *wa, *wb;
+  uint64_t m, k, n, kp;  // kp: k rounded up to 64 (a row of a plane)
+  __half *pa, *pb;       // [da][m][kp], [db][n][kp]
+  uint32_t row_runs;     // A: warp-runs (32 groups of 8 fields) per row
+  uint32_t blocks_a;     // CTAs [0, blocks_a) write A's planes, the rest B's
+  uint32_t tiles_k;      // B: 64 x 64 tiles along k
+};
+
+// A's planes: 8 fields of a row per lane, one 16-byte store per digit.
+template <int B>
+__device__ __forceinline__ void planes_a(const PlaneArgs& a, const Split& sp) {
+  const int sgn = a.ha->is_signed, lane = threadIdx.x % 32;
+  const bool small = sp.wa <= 9;
+  const uint64_t items = a.m * a.row_runs;
+  for (uint64_t it = (uint64_t)blockIdx.x * 8 + threadIdx.x / 32; it < items;
+       it += (uint64_t)a.blocks_a * 8) {
+    const uint64_t i = items >> 32 ? it / a.row_runs : (uint32_t)it / a.row_runs;
+    const uint64_t kk = 8 * ((it - i * a.row_runs) * 32 + lane);
+    if (kk >= a.kp) continue;
+    int v[8];
+    decode8<B>(a.wa, i * a.k + kk, kk < a.k ? (int)umin(8, a.k - kk) : 0, sgn, v);
+    __half* dst = a.pa + i * a.kp + kk;
+    for (int l = 0; l < sp.da; ++l, dst += a.m * a.kp) {
+      int d[8];
 #pragma unroll
-        for (int l = 0; l < L; ++l) out[l] = plane_bytes8<L>(wg, l, sgn && l == L - 1);
-      } else {
-#pragma unroll
-        for (int l = 0; l < L; ++l) out[l] = make_uint2(0u, 0u);
-      }
-#pragma unroll
-      for (int l = 0; l < L; ++l)
-        *reinterpret_cast<uint2*>(planes + l * plane + i * k_pad + kk) = out[l];
+      for (int j = 0; j < 8; ++j) d[j] = l + 1 < sp.da ? take_digit(v[j], sp.wa) : v[j];
+      *reinterpret_cast<uint4*>(dst) =
+          make_uint4(half2_bits(d[0], d[1], small), half2_bits(d[2], d[3], small),
+                     half2_bits(d[4], d[5], small), half2_bits(d[6], d[7], small));
     }
   }
 }
 
-// A (m x k, row-major) -> planes [L][m_pad][k_pad] of e4m3 digits.
-__global__ void k_limbs_a(const ccm_header* out, const ccm_header* h, const uint32_t* __restrict__ w,
-                          uint64_t m, uint64_t k, uint64_t m_pad, uint64_t k_pad, int L,
-                          uint8_t* __restrict__ planes) {
-  if (out->status != CCM_OK) return;
-  const int b = h->width, sgn = h->is_signed;
-  if (b == 4 * L && k % 8 == 0) {  // nibble-aligned fields
-    switch (L) {
-      case 1: limbs_a_nibbles<1>(w, sgn, m, k, m_pad, k_pad, planes); return;
-      case 2: limbs_a_nibbles<2>(w, sgn, m, k, m_pad, k_pad, planes); return;
-      case 3: limbs_a_nibbles<3>(w, sgn, m, k, m_pad, k_pad, planes); return;
-      case 4: limbs_a_nibbles<4>(w, sgn, m, k, m_pad, k_pad, planes); return;
+// B's planes: a 64 (k) x 64 (n) tile per CTA; a thread decodes 8 fields of two
+// rows of B and writes them as (k, k + 1) pairs into a transposed shared tile,
+// whose rows (64 k of one column) leave as 16-byte stores.
+template <int B>
+__device__ __forceinline__ void planes_b(const PlaneArgs& a, const Split& sp,
+                                         uint32_t (*tile)[33]) {
+  const int sgn = a.hb->is_signed, tid = threadIdx.x;
+  const bool small = sp.wb <= 9;
+  const uint32_t t = blockIdx.x - a.blocks_a;
+  const uint64_t k0 = (uint64_t)(t % a.tiles_k) * 64, j0 = (uint64_t)(t / a.tiles_k) * 64;
+  const int cols = (int)umin(64, a.n - j0);
+  const int g8 = 8 * (tid % 8), kpair = tid / 8, cnt = min(8, cols - g8);
+  const uint64_t row = k0 + 2 * kpair;
+  int v0[8], v1[8];
+  decode8<B>(a.wb, row * a.n + j0 + g8, row < a.k ? cnt : 0, sgn, v0);
+  decode8<B>(a.wb, (row + 1) * a.n + j0 + g8, row + 1 < a.k ? cnt : 0, sgn, v1);
+  const int col = tid / 4, q = tid % 4;
+  __half* dst = a.pb + (j0 + col) * a.kp + k0 + 16 * q;
+  for (int l = 0; l < sp.db; ++l, dst += a.n * a.kp) {
+    const bool last = l + 1 == sp.db;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int x = last ? v0[j] : take_digit(v0[j], sp.wb);
+      const int y = last ? v1[j] : take_digit(v1[j], sp.wb);
+      tile[g8 + j][kpair] = half2_bits(x, y, small);
+    }
+    __syncthreads();
+    if (col < cols) {
+      const uint32_t* src = &tile[col][8 * q];
+      reinterpret_cast<uint4*>(dst)[0] = make_uint4(src[0], src[1], src[2], src[3]);
+      reinterpret_cast<uint4*>(dst)[1] = make_uint4(src[4], src[5], src[6], src[7]);
+    }
+    __syncthreads();
+  }
+}
+
+#define CCM_TC_WIDTHS(M)                                                                       \
+  M(1) M(2) M(3) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12) M(13) M(14) M(15) M(16) M(17) \
+  M(18) M(19) M(20) M(21) M(22) M(23) M(24) M(25) M(26) M(27) M(28) M(29) M(30) M(31)
+
+// Both operands' planes in one launch.  The bytes are b/8 in and 2 d out per
+// field; what is left beside them is the cutting of the fields, so the widths
+// are compile-time bodies chosen from the headers.
+__global__ void __launch_bounds__(256) k_planes(const __grid_constant__ PlaneArgs a) {
+  __shared__ uint32_t tile[64][33];
+  ax::grid_dep_launch();
+  ax::grid_dep_wait();
+  if (a.out->status != CCM_OK) return;
+  const Split sp = split_of(a.ha, a.hb);
+  if (blockIdx.x < a.blocks_a) {
+    switch (a.ha->width) {
+#define CCM_TC_A(B) \
+  case B: planes_a<B>(a, sp); break;
+      CCM_TC_WIDTHS(CCM_TC_A)
+#undef CCM_TC_A
+      default: break;
+    }
+  } else {
+    switch (a.hb->width) {
+#define CCM_TC_B(B) \
+  case B: planes_b<B>(a, sp, tile); break;
+      CCM_TC_WIDTHS(CCM_TC_B)
+#undef CCM_TC_B
       default: break;
     }
   }
-  const uint64_t quads = m_pad * k_pad / 4;
-  const uint64_t plane = m_pad * k_pad;
-  for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < quads;
-       q += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t e0 = 4 * q, i = e0 / k_pad, kk = e0 % k_pad;
-    int64_t v[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-      v[t] = (i < m && kk + t < k) ? decode_field(w, i * k + kk + t, b, sgn) : 0;
-    for (int l = 0; l < L; ++l) {
-      uint32_t word = 0;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) word |= (uint32_t)e4m3_of_digit(digit(v[t], l, L)) << (8 * t);
-      *reinterpret_cast<uint32_t*>(planes + l * plane + e0) = word;
-    }
-  }
-}
-
-// B (k x n, row-major) -> planes [L][n_pad][k_pad] (transposed, K-major).
-__global__ void __launch_bounds__(256) k_limbs_bt(const ccm_header* out, const ccm_header* h,
-                                                  const uint32_t* __restrict__ w, uint64_t k,
-                                                  uint64_t n, uint64_t n_pad, uint64_t k_pad, int L,
-                                                  uint8_t* __restrict__ planes) {
-  __shared__ uint8_t tile[4][32][64 + 4];  // [digit][j][kk]
-  if (out->status != CCM_OK) return;
-  const int b = h->width, sgn = h->is_signed;
-  const uint64_t plane = n_pad * k_pad;
-  const uint64_t tiles_k = k_pad / 64, tiles_n = n_pad / 32;
-  // nibble-aligned fields (b = 4L <= 16) and rows of whole 8-field groups:
-  // thread t reads fields j = 8 (t % 4) .. + 7 of row kk = t / 4 of the tile
-  const bool nib = b == 4 * L && L <= 4 && n % 8 == 0;
-  for (uint64_t t = blockIdx.x; t < tiles_k * tiles_n; t += gridDim.x) {
-    const uint64_t k0 = (t % tiles_k) * 64, j0 = (t / tiles_k) * 32;
-    for (int l0 = 0; l0 < L; l0 += 4) {
-      if (nib) {
-        const int kk = threadIdx.x / 4, jg = 8 * (threadIdx.x % 4);
-        const uint64_t gk = k0 + kk, gj = j0 + jg;
-        uint2 bytes[4] = {};
-        const bool live = gk < k && gj < n;
-        switch (L) {
-#define CCM_TC_NIB(LL)                                                           \
-  case LL:                                                                       \
-    if (live) {                                                                  \
-      uint32_t wg[LL];                                                           \
-      load_group8<LL>(w, gk * n + gj, wg);                                       \
-      _Pragma("unroll") for (int l = 0; l < LL; ++l) bytes[l] =                  \
-          plane_bytes8<LL>(wg, l, sgn && l == LL - 1);                           \
-    }                                                                            \
-    break;
-          CCM_TC_NIB(1) CCM_TC_NIB(2) CCM_TC_NIB(3) CCM_TC_NIB(4)
-#undef CCM_TC_NIB
-          default: break;
-        }
-        for (int l = 0; l < L; ++l) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            tile[l][jg + q][kk] = (uint8_t)((q < 4 ? bytes[l].x : bytes[l].y) >> (8 * (q & 3)));
-        }
-      } else {
-        // read: thread covers (kk = threadIdx.x / 32 + 8 r, j = threadIdx.x % 32)
-        for (int r = 0; r < 8; ++r) {
-          const int kk = threadIdx.x / 32 + 8 * r, j = threadIdx.x % 32;
-          const uint64_t gk = k0 + kk, gj = j0 + j;
-          const int64_t v = (gk < k && gj < n) ? decode_field(w, gk * n + gj, b, sgn) : 0;
-          for (int l = l0; l < L && l < l0 + 4; ++l)
-            tile[l - l0][j][kk] = e4m3_of_digit(digit(v, l, L));
-        }
-      }
-      __syncthreads();
-      // write: 32 rows (j) x 64 bytes per digit plane, 16 bytes per thread
-      for (int l = l0; l < L && l < l0 + 4; ++l) {
-        const int j = threadIdx.x / 4, part = threadIdx.x % 4;
-        if (threadIdx.x < 128) {
-          const uint8_t* src = &tile[l - l0][j][16 * part];
-          uint4 v;
-          v.x = src[0] | src[1] << 8 | src[2] << 16 | (uint32_t)src[3] << 24;
-          v.y = src[4] | src[5] << 8 | src[6] << 16 | (uint32_t)src[7] << 24;
-          v.z = src[8] | src[9] << 8 | src[10] << 16 | (uint32_t)src[11] << 24;
-          v.w = src[12] | src[13] << 8 | src[14] << 16 | (uint32_t)src[15] << 24;
-          *reinterpret_cast<uint4*>(planes + l * plane + (j0 + j) * k_pad + k0 + 16 * part) = v;
-        }
-      }
-      __syncthreads();
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
-// PTX wrappers (sm_100+ family: tcgen05, TMA, mbarrier)
+// PTX wrappers (tcgen05 with CTA pairs, TMA, cluster mbarriers)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %cluster_ctarank;\n" : "=r"(r));
+  return r;
 }
 
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count));
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(p));
+  return p != 0;
 }
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
-               "r"(bytes)
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::
+                   : "memory");
+}
+
+// The shared::cluster address of `p` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+  return r;
+}
+
+__device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr)
                : "memory");
 }
 
-__device__ __forceinline__ uint64_t globaltimer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %globaltimer;\n" : "=l"(t));
-  return t;
+__device__ __forceinline__ uint32_t ld_remote(uint32_t cluster_addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
 }
 
-// Bounded wait for the phase with parity `parity`: gives up (returns false)
-// after about two seconds, or after kSpinLimit polls.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t addr = smem_u32(bar);
-  uint64_t t0 = 0;
-  for (uint32_t it = 0; it < kSpinLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if ((it & 1023) == 0) {
-      const uint64_t now = globaltimer_ns();
-      if (it == 0)
-        t0 = now;
-      else if (now - t0 > 2000000000ull)
-        return false;
-    }
-  }
-  return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
-                                            int y) {
+// kSub blocks of k from block x on, rows from y on, of plane z; the bytes are
+// counted on the leader's barrier.
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar,
+                                              int x, int y, int z) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];\n" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(0), "r"(y), "r"(x), "r"(z)
       : "memory");
 }
 
@@ -352,69 +338,84 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor: kind::f8f6f4, A = B = e4m3, D = f32, both K-major.
-__host__ __device__ constexpr uint32_t idesc_e4m3_f32(int m, int n) {
+// Instruction descriptor: kind::f16, A = B = f16, D = f32, both K-major.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int m, int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_e4m3(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+// Arrives on `bar` (same offset) in both CTAs of the pair when the MMAs
+// issued so far have completed.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-          smem_u32(bar))
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;\n" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
       : "memory");
 }
 
-// tcgen05.ld of 32 columns without the wait (several in flight, then
-// tmem_ld_wait before the registers are used).
-__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+__device__ __forceinline__ void tmem_fence_before() {
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+}
+__device__ __forceinline__ void tmem_fence_after() {
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
 
+// ---------------------------------------------------------------------------
+// The product kernel
+// ---------------------------------------------------------------------------
 struct MmArgs {
-  ccm_header* out;      // C header: status, width statistics
-  int64_t* c;           // int64 C, m x n row-major
+  ccm_header* out;  // C header: status, width statistics
+  const ccm_header *ha, *hb;
+  void* c;          // C, m x n row-major, int64 or int32
   uint64_t m, n;
-  uint32_t k_blocks;    // k_pad / kBK
-  uint32_t a_rows_pad;  // rows per A digit plane (m_pad)
-  uint32_t b_rows_pad;  // rows per B digit plane (n_pad)
-  uint32_t tiles_n;     // n_pad / bn
-  uint32_t tiles_m;     // m_pad / kBM
-  int L;
-  int c32;              // 1: C is written as int32 (the output capacity bounds its width by 31)
+  uint32_t k_blocks;
+  uint32_t tiles_m, tiles_n;
+  int c32;          // 1: C is stored as int32 (the output capacity bounds its width by 31)
+};
+
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 32 * (4 + kEpiWarps);  // (two warps idle: registers are granted per four warps)
+
+// Geometry of one instance.  Acc64: C needs more than 32 bits, so a thread
+// holds 64-bit accumulators and the tile is at most 128 columns wide.
+template <int BN, bool kAcc64>
+struct Geo {
+  static constexpr int kHalf = BN / 2;                 // columns per epilogue half
+  static constexpr int kCCols = !kAcc64 && kHalf % 32 == 0 ? 32 : 16;  // columns stored at a time
+  // blocks of k per stage: a stage costs about 380 cycles of barrier round
+  // trips in the producer and the issuer, a block BN * 2 cycles of MMA
+  static constexpr int kSub = BN > 128 ? 1 : 2;
+  static constexpr uint32_t kATile = 128 * kBK * 2;    // bytes per CTA and block of k
+  static constexpr uint32_t kBTile = (BN / 2) * kBK * 2;
+  static constexpr uint32_t kBOff = kSub * kATile;     // B's blocks behind A's
+  static constexpr uint32_t kStage = kSub * (kATile + kBTile);
+  static constexpr uint32_t kCStage = 32 * (kCCols + 1) * (kAcc64 ? 8 : 4);  // per epilogue warp
+  static constexpr int kBufs = BN > 128 ? 2 : 4;       // accumulators in tensor memory
+  static constexpr uint32_t kBufCols = 512 / kBufs;
+  static constexpr int kStages = (int)((224 * 1024 - kEpiWarps * kCStage) / kStage) > 8
+                                     ? 8
+                                     : (int)((224 * 1024 - kEpiWarps * kCStage) / kStage);
+  static constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + kEpiWarps * kCStage;
 };
 
 // Output tile t (grouped raster): consecutive tiles sweep the tile columns
@@ -429,374 +430,469 @@ __device__ __forceinline__ void tile_coords(uint32_t t, uint32_t tiles_m, uint32
   tn = in_group / gm;
 }
 
-// Persistent, warp-specialised: one CTA per SM walks the output tiles t =
-// blockIdx.x, + gridDim.x, ...  Warp 0 (one thread) streams the digit-plane
-// tiles of every k block of every tile through the S-stage ring (TMA,
-// mbarriers); warp 1 allocates tensor memory and one of its threads issues
-// the MMAs of tile i into accumulator set i % accs, once the epilogue has
-// emptied that set; warps 2-5 (tensor-memory lane quadrants 2, 3, 0, 1) read
-// the classes of each finished tile, combine them exactly and store C.  The
-// producer runs on into the next tile's loads while the current one is
-// finished, and with two accumulator sets (one digit) the next tile's MMAs
-// run during the previous tile's epilogue.
-constexpr int kThreadsP = 192;
+// acc += run << shift for 16 columns: the run's sums are integers of at most
+// 2^24, so the conversion is exact.
+__device__ __forceinline__ void add_run(const uint32_t (&r)[16], int shift, uint32_t* acc) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) acc[j] += (uint32_t)__float2int_rn(__uint_as_float(r[j])) << shift;
+}
+__device__ __forceinline__ void add_run(const uint32_t (&r)[16], int shift,
+                                        unsigned long long* acc) {
+  if (shift <= 30) {  // one 32 x 32 -> 64-bit multiply-add per column
+    const int mul = 1 << shift;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      acc[j] += (unsigned long long)((long long)__float2int_rn(__uint_as_float(r[j])) * mul);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      acc[j] += (unsigned long long)((long long)__float2int_rn(__uint_as_float(r[j]))) << shift;
+  }
+}
 
-template <int L>
-__global__ void __launch_bounds__(kThreadsP, 1)
-    k_mm_tc(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-            MmArgs args) {
-  constexpr Geo G = geometry(L);
-  constexpr int BN = G.bn, S = G.stages, C = G.classes, NACC = G.accs;
-  constexpr uint32_t ACC_COLS = (uint32_t)(C * BN);          // columns of one accumulator set
-  constexpr uint32_t A_TILE = kBM * kBK, B_TILE = BN * kBK;  // bytes per digit plane tile
-  constexpr uint32_t STAGE = L * (A_TILE + B_TILE);
+// One warp's 32 rows x kHalf columns of C, from one row per lane to rows of
+// consecutive lanes: through a transposing tile, kCCols columns at a time.
+template <int BN, bool kAcc64, typename T, typename UAcc, typename Acc>
+__device__ __forceinline__ void store_tile(const UAcc (&acc)[BN / 2], Acc* st, int lane, T* c,
+                                           uint64_t row0, uint64_t col0, uint64_t m, uint64_t n) {
+  constexpr int W = Geo<BN, kAcc64>::kCCols, kRows = 32 / W;
+  const int r0 = lane / W, cl = lane % W;
+  const int rows = row0 < m ? (int)umin(32, m - row0) : 0;
+#pragma unroll
+  for (int c0 = 0; c0 < BN / 2; c0 += W) {
+#pragma unroll
+    for (int j = 0; j < W; ++j) st[lane * (W + 1) + j] = (Acc)acc[c0 + j];
+    __syncwarp();
+    const uint64_t col = col0 + c0 + cl;
+    if (col < n) {
+      T* dst = c + (row0 + r0) * n + col;
+      const Acc* src = st + r0 * (W + 1) + cl;
+#pragma unroll 8
+      for (int r = 0; r < 32; r += kRows) {
+        if (r + r0 < rows) *dst = (T)src[r * (W + 1)];
+        dst += kRows * n;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+template <int BN, bool kAcc64>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    k_mm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+         const __grid_constant__ MmArgs args) {
+  using G = Geo<BN, kAcc64>;
+  using Acc = typename std::conditional<kAcc64, long long, int>::type;
+  using UAcc = typename std::make_unsigned<Acc>::type;  // (sums wrap: only the total must fit)
+  constexpr int S = G::kStages;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
-  __shared__ uint64_t full_bar[S], empty_bar[S], acc_full[NACC], acc_empty[NACC];
+  __shared__ uint64_t full_bar[S], empty_bar[S], acc_full[G::kBufs], acc_empty[G::kBufs];
   __shared__ uint32_t tmem_base_s;
-  __shared__ int skip_s;
+  __shared__ __align__(4) Split split_s;
   __shared__ volatile int abort_s;
-  __shared__ uint32_t issued_s;  // k blocks whose loads the producer issued (all tiles)
+  __shared__ uint32_t issued_s;  // stages whose loads this CTA issued
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  // one read of the status for the whole CTA (another CTA may change it)
-  if (threadIdx.x == 0) skip_s = args.out->status != CCM_OK;
-  __syncthreads();
-  if (skip_s) return;
-  const uint32_t tiles = args.tiles_m * args.tiles_n;
-  const uint32_t nk = args.k_blocks;
-
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
+  const uint32_t rank = cluster_rank();
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
     }
-    for (int a = 0; a < NACC; ++a) {
+    for (int a = 0; a < G::kBufs; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 4);  // one arrival per epilogue warp
+      mbar_init(&acc_empty[a], 2 * kEpiWarps);  // the epilogue warps of both CTAs
     }
     abort_s = 0;
     issued_s = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    ax::mbar_init_fence();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      smem_u32(&tmem_base_s)),
-                 "r"((uint32_t)G.tmem_cols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  ax::grid_dep_launch();
+  ax::grid_dep_wait();
+  // the leader's reading of the status and the widths decides for the pair
+  // (another CTA may set the status meanwhile)
+  if (rank == 0 && threadIdx.x == 0) {
+    split_s = split_of(args.ha, args.hb);
+    if (args.out->status != CCM_OK) split_s.da = 0;
+  }
+  tmem_fence_before();
+  cluster_sync();
+  tmem_fence_after();
   const uint32_t tmem = tmem_base_s;
+  const uint32_t sw = ld_remote(map_rank(&split_s, 0));
+  const Split sp{(uint8_t)sw, (uint8_t)(sw >> 8), (uint8_t)(sw >> 16), (uint8_t)(sw >> 24)};
+  const uint32_t tiles = sp.da ? args.tiles_m * args.tiles_n : 0;
+  const uint32_t nk = (args.k_blocks + G::kSub - 1) / G::kSub;  // stages along k
+  const uint32_t pairs = sp.da * sp.db;
+  const uint32_t run = min((uint32_t)(sp.run() / (kBK * G::kSub)), nk);  // stages per flush
+  const uint32_t first = blockIdx.x / 2, step = gridDim.x / 2;
 
-  uint64_t orv = 0;
-  uint32_t neg = 0;
+  // Producer and issuer run as whole warps, one elected lane issuing, so that
+  // addresses and descriptors stay in uniform registers, and nothing but the
+  // stage's barrier is touched per k block: every further access to shared
+  // memory costs a hundred cycles or so of a loop that has 512 (at BN = 256).
+  // Issued from a single-lane branch with an abort flag read per k block, a
+  // k block took 730-780 cycles whatever BN was.
   if (warp == 0) {
-    if (lane == 0) {
-      // TMA producer over every k block of every tile of this CTA
-      uint32_t g = 0;
-      for (uint32_t t = blockIdx.x; t < tiles && !abort_s; t += gridDim.x) {
-        uint32_t tm, tn;
-        tile_coords(t, args.tiles_m, args.tiles_n, tm, tn);
-        for (uint32_t kb = 0; kb < nk; ++kb, ++g) {
-          const int s = g % S;
-          if (g >= (uint32_t)S && !mbar_wait(&empty_bar[s], ((g / S) - 1) & 1)) {
-            abort_s = 1;
-            break;
-          }
-          if (abort_s) break;
-          uint8_t* st = smem + s * STAGE;
-          mbar_expect_tx(&full_bar[s], STAGE);
-          for (int l = 0; l < L; ++l) {
-            tma_load_2d(st + l * A_TILE, &tm_a, &full_bar[s], kb * kBK,
-                        l * args.a_rows_pad + tm * kBM);
-            tma_load_2d(st + L * A_TILE + l * B_TILE, &tm_b, &full_bar[s], kb * kBK,
-                        l * args.b_rows_pad + tn * BN);
-          }
-          issued_s = g + 1;
-        }
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      constexpr uint32_t idesc = idesc_e4m3_f32(kBM, BN);
-      uint32_t g = 0, i = 0;
-      bool ok = true;
-      for (uint32_t t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
-        const uint32_t a = i % NACC;
-        if (i >= (uint32_t)NACC && !mbar_wait(&acc_empty[a], ((i / NACC) - 1) & 1)) {
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const uint32_t acc0 = tmem + a * ACC_COLS;
-        uint32_t started = 0;  // classes already holding a partial sum
-        for (uint32_t kb = 0; kb < nk; ++kb, ++g) {
-          const int s = g % S;
-          if (abort_s || !mbar_wait(&full_bar[s], (g / S) & 1)) {
+    const uint32_t full0 = __shfl_sync(0xffffffffu, map_rank(&full_bar[0], 0), 0);
+    const uint32_t smem0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+    uint32_t s = 0, parity = 1, issued = 0;
+    bool ok = true;
+    for (uint32_t t = first; t < tiles && ok; t += step) {
+      uint32_t tm, tn;
+      tile_coords(t, args.tiles_m, args.tiles_n, tm, tn);
+      const int ya = tm * kBM + rank * 128, yb = tn * BN + rank * (BN / 2);
+      for (uint32_t p = 0; p < pairs && ok; ++p) {
+        const int l = p / sp.db, q = p % sp.db;
+        if (abort_s) ok = false;
+        for (uint32_t kb = 0; kb < nk && ok; ++kb) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], parity))) {
             ok = false;
             break;
           }
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-          const uint32_t st = smem_u32(smem + s * STAGE);
-#pragma unroll
-          for (int l = 0; l < L; ++l) {
-#pragma unroll
-            for (int mm = 0; mm < L; ++mm) {
-              const int c = l + mm;
-              const uint32_t a0 = st + l * A_TILE, b0 = st + L * A_TILE + mm * B_TILE;
-#pragma unroll
-              for (int kk = 0; kk < kBK / 32; ++kk) {
-                const uint32_t acc = ((started >> c) & 1u) | (kk > 0 ? 1u : 0u);
-                mma_e4m3(acc0 + c * BN, smem_desc_sw128(a0 + 32 * kk),
-                         smem_desc_sw128(b0 + 32 * kk), idesc, acc);
-              }
-              started |= 1u << c;
-            }
+          if (elect_one()) {
+            if (rank == 0) ax::mbar_expect_tx(&full_bar[s], 2 * G::kStage);
+            tma_load_pair(smem0 + s * G::kStage, &map_a, full0 + 8 * s, G::kSub * kb, ya, l);
+            tma_load_pair(smem0 + s * G::kStage + G::kBOff, &map_b, full0 + 8 * s, G::kSub * kb, yb, q);
           }
-          mma_commit(&empty_bar[s]);  // frees the stage once these MMAs have read it
+          __syncwarp();
+          ++issued;
+          if (++s == (uint32_t)S) {
+            s = 0;
+            parity ^= 1;
+          }
         }
-        mma_commit(&acc_full[a]);  // (also when giving up: the MMAs issued so far complete)
+      }
+    }
+    if (lane == 0) issued_s = issued;
+    // the leader's commits still on their way to this CTA's barriers
+    for (uint32_t x = issued > (uint32_t)S ? issued - S : 0; x < issued && ok; ++x)
+      ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[x % S], (x / S) & 1));
+    if (!ok) abort_s = 1;
+  } else if (warp == 1) {
+    if (rank == 0) {
+      constexpr uint32_t idesc = idesc_f16_f32(kBM, BN);
+      const uint32_t smem0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+      const uint32_t tmem0 = __shfl_sync(0xffffffffu, tmem, 0);
+      uint32_t s = 0, parity = 0, f = 0;  // stage and its phase; runs
+      bool ok = true;
+      for (uint32_t t = first; t < tiles && ok; t += step) {
+        for (uint32_t p = 0; p < pairs && ok; ++p) {
+          for (uint32_t k0 = 0; k0 < nk && ok; k0 += run, ++f) {
+            const uint32_t buf = f % G::kBufs;
+            if (abort_s || !__all_sync(0xffffffffu,
+                                       mbar_wait(&acc_empty[buf], ((f / G::kBufs) & 1) ^ 1))) {
+              ok = false;
+              break;
+            }
+            tmem_fence_after();
+            const uint32_t acc = tmem0 + buf * G::kBufCols;
+            const uint32_t k1 = k0 + run < nk ? k0 + run : nk;
+            for (uint32_t kb = k0; kb < k1; ++kb) {
+              if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], parity))) {
+                ok = false;
+                break;
+              }
+              tmem_fence_after();
+              const uint64_t da = smem_desc_sw128(smem0 + s * G::kStage);
+              const uint64_t db = smem_desc_sw128(smem0 + s * G::kStage + G::kBOff);
+              if (elect_one()) {
+#pragma unroll
+                for (int kk = 0; kk < 4 * G::kSub; ++kk) {
+                  // 32 bytes further along k; the second block is a tile on
+                  const uint32_t in = 2 * (kk % 4), blk = kk / 4;
+                  mma_f16_pair(acc, da + in + blk * (G::kATile / 16), db + in + blk * (G::kBTile / 16),
+                               idesc, (kb > k0 || kk > 0) ? 1u : 0u);
+                }
+                mma_commit_pair(&empty_bar[s]);  // frees the stage in both CTAs
+              }
+              __syncwarp();
+              if (++s == (uint32_t)S) {
+                s = 0;
+                parity ^= 1;
+              }
+            }
+            if (elect_one())
+              mma_commit_pair(&acc_full[buf]);  // (also when giving up: what was issued completes)
+            __syncwarp();
+          }
+        }
       }
       if (!ok) abort_s = 1;
     }
-  } else {
-    // epilogue: tensor-memory lane quadrant q of every finished tile
-    const int q = warp % 4;
+  } else if (warp >= 4) {
+    // epilogue: tensor-memory lane quadrant q, column half h of every tile
+    const int ew = warp - 4, q = warp % 4, h = ew / 4;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    uint32_t i = 0;
-    for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
-      const uint32_t a = i % NACC;
-      // (one decision for the whole warp: the tensor-memory loads are warp-wide)
-      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[a], (i / NACC) & 1))) {
+    uint8_t* cst = smem + S * G::kStage + ew * G::kCStage;
+    UAcc orv = 0, sgn = 0;
+    uint32_t f = 0;
+    bool ok = true;
+    for (uint32_t t = first; t < tiles && ok; t += step) {
+      UAcc acc[G::kHalf];
+#pragma unroll
+      for (int j = 0; j < G::kHalf; ++j) acc[j] = 0;
+      for (uint32_t p = 0; p < pairs && ok; ++p) {
+        const int shift = sp.wa * (int)(p / sp.db) + sp.wb * (int)(p % sp.db);
+        for (uint32_t k0 = 0; k0 < nk; k0 += run, ++f) {
+          const uint32_t buf = f % G::kBufs;
+          // (one decision for the whole warp: the tensor-memory loads are warp-wide)
+          if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (f / G::kBufs) & 1)) ||
+              __any_sync(0xffffffffu, abort_s != 0)) {
+            ok = false;
+            break;
+          }
+          tmem_fence_after();
+          const uint32_t src = tmem + lane_base + buf * G::kBufCols + h * G::kHalf;
+#pragma unroll
+          for (int c = 0; c < G::kHalf; c += 16) {
+            uint32_t r[16];
+            tmem_ld16(src + c, r);
+            tmem_ld_wait();
+            add_run(r, shift, &acc[c]);
+          }
+          // this accumulator has been read: the run after next may start
+          tmem_fence_before();
+          __syncwarp();
+          if (lane == 0) arrive_remote(map_rank(&acc_empty[buf], 0));
+        }
+      }
+      if (!ok) {
         abort_s = 1;
         break;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      if (__any_sync(0xffffffffu, abort_s != 0)) break;
       uint32_t tm, tn;
       tile_coords(t, args.tiles_m, args.tiles_n, tm, tn);
-      const uint64_t row = (uint64_t)tm * kBM + q * 32 + lane;
-      const uint32_t acc0 = tmem + lane_base + a * ACC_COLS;
-#pragma unroll 1
-      for (int col0 = 0; col0 < BN; col0 += 32) {
-        int64_t acc[32];
+      const uint64_t row0 = (uint64_t)tm * kBM + rank * 128 + q * 32;
+      const uint64_t col0 = (uint64_t)tn * BN + h * G::kHalf;
+      // (rows and columns outside C are products of zero fill: they add nothing)
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0;
-        if constexpr (C <= 3) {
-          // two classes' loads in flight at a time (for more classes the
-          // registers this takes cost more than the overlap gains)
-#pragma unroll 1
-          for (int c = 0; c < C; c += 2) {
-            uint32_t r0[32], r1[32];
-            tmem_ld32_async(acc0 + c * BN + col0, r0);
-            if (c + 1 < C) tmem_ld32_async(acc0 + (c + 1) * BN + col0, r1);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              acc[j] += (int64_t)__float2ll_rn(__uint_as_float(r0[j])) * (int64_t)(1ll << (4 * c));
-            if (c + 1 < C) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                acc[j] += (int64_t)__float2ll_rn(__uint_as_float(r1[j])) *
-                          (int64_t)(1ll << (4 * (c + 1)));
-            }
-          }
-        } else {
-#pragma unroll 1
-          for (int c = 0; c < C; ++c) {
-            uint32_t r[32];
-            tmem_ld32(acc0 + c * BN + col0, r);
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              acc[j] += (int64_t)__float2ll_rn(__uint_as_float(r[j])) * (int64_t)(1ll << (4 * c));
-          }
-        }
-        const uint64_t col = (uint64_t)tn * BN + col0;
-        if (row < args.m) {
-          int64_t* dst = args.c + row * args.n + col;
-          int32_t* dst32 = reinterpret_cast<int32_t*>(args.c) + row * args.n + col;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (col + j < args.n) {
-              if (args.c32)
-                dst32[j] = (int32_t)acc[j];  // (statistics from the exact value below)
-              else
-                dst[j] = acc[j];
-              orv |= fold(acc[j]);
-              neg |= (uint32_t)(acc[j] < 0);
-            }
-          }
-        }
+      for (int j = 0; j < G::kHalf; ++j) {
+        orv |= (UAcc)((Acc)acc[j] ^ ((Acc)acc[j] >> (sizeof(Acc) * 8 - 1)));
+        sgn |= acc[j];
       }
-      // this set's tensor memory has been read: the MMAs of tile i + accs may start
-      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-      __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acc_empty[a]))
-                     : "memory");
+      if (args.c32)
+        store_tile<BN, kAcc64, int32_t>(acc, reinterpret_cast<Acc*>(cst), lane,
+                                        reinterpret_cast<int32_t*>(args.c), row0, col0, args.m,
+                                        args.n);
+      else
+        store_tile<BN, kAcc64, int64_t>(acc, reinterpret_cast<Acc*>(cst), lane,
+                                        reinterpret_cast<int64_t*>(args.c), row0, col0, args.m,
+                                        args.n);
     }
-    orv = warp_or64(orv);
-    neg = __reduce_or_sync(0xffffffffu, neg);
+    const uint64_t orv64 = warp_or64((uint64_t)orv);
+    const uint32_t neg = __any_sync(0xffffffffu, (Acc)sgn < 0);
     if (lane == 0) {
-      if (orv) atomicOr(reinterpret_cast<unsigned long long*>(&args.out->stat_or),
-                        (unsigned long long)orv);
+      if (orv64) atomicOr(reinterpret_cast<unsigned long long*>(&args.out->stat_or),
+                          (unsigned long long)orv64);
       if (neg) atomicOr(&args.out->stat_neg, 1u);
     }
   }
   __syncwarp();
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  tmem_fence_before();
   __syncthreads();
-  if (abort_s && threadIdx.x == 0) {
-    // a wait gave up: let the copies already issued land (bounded) before the
-    // CTA's shared memory is released, and report it
-    const uint32_t issued = issued_s;
-    for (uint32_t g = issued > (uint32_t)S ? issued - S : 0; g < issued; ++g)
-      mbar_wait(&full_bar[g % S], (g / S) & 1);
-    set_status(args.out, CCM_E_TIMEOUT);
+  if (threadIdx.x == 0) {
+    // the copies of both CTAs land on the leader's barriers: all of them have
+    // (at once) unless a wait gave up, and then this waits for them (bounded)
+    // before shared memory is released
+    if (rank == 0) {
+      const uint32_t issued = issued_s;
+      for (uint32_t g = issued > (uint32_t)S ? issued - S : 0; g < issued; ++g)
+        if (!mbar_wait(&full_bar[g % S], (g / S) & 1)) break;
+    }
+    if (abort_s) set_status(args.out, CCM_E_TIMEOUT);
   }
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  cluster_sync();
+  tmem_fence_after();
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"((uint32_t)G.tmem_cols));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u));
   }
 }
 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-struct Plan {
-  int L;
-  uint64_t m_pad, n_pad, k_pad;
-  size_t a_bytes, b_bytes;
-};
-
-Plan plan_for(uint64_t m, uint64_t k, uint64_t n, int L) {
-  Geo g = geometry(L);
-  Plan p;
-  p.L = L;
-  p.m_pad = round_up(m, kBM);
-  p.n_pad = round_up(n, (uint64_t)g.bn);
-  p.k_pad = round_up(k, kBK);
-  p.a_bytes = (size_t)L * p.m_pad * p.k_pad;
-  p.b_bytes = (size_t)L * p.n_pad * p.k_pad;
-  return p;
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
     cudaDriverEntryPointQueryResult q;
     void* p = nullptr;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
                                          &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
+      return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    return nullptr;
+  }();
   return fn;
 }
 
-bool make_map(CUtensorMap* map, void* base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+// Planes [d][rows][kp], as blocks of 64 along k; rows past the end and an odd
+// last block are read as zero.
+bool make_map(CUtensorMap* map, void* base, uint64_t kp, uint64_t rows, int d, uint32_t box_rows,
+              uint32_t box_blocks) {
   auto fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[2] = {inner, rows};
-  cuuint64_t strides[1] = {inner};
-  cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr,
+  cuuint64_t dims[4] = {64, rows, kp / 64, (cuuint64_t)d};
+  cuuint64_t strides[3] = {kp * 2, 128, rows * kp * 2};
+  cuuint32_t box[4] = {64, box_rows, box_blocks, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, base, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int digits_for(int bmax) { return (bmax + 3) / 4; }
+// Most digits per operand over every pair of widths up to (ba, bb) and both
+// sign modes (the widths and signs themselves are only known on the GPU);
+// {0, 0} when some of them has no split.
+struct DigitBound {
+  uint8_t da, db;
+};
+DigitBound digit_bound(int ba, int bb) {
+  DigitBound d{0, 0};
+  if (ba < 1 || bb < 1 || ba + 1 > kMaxE || bb + 1 > kMaxE) return d;
+  for (int ea = 1; ea <= ba + 1; ++ea)
+    for (int eb = 1; eb <= bb + 1; ++eb) {
+      const Split& s = kSplits.at[ea][eb];
+      if (!s.da) return DigitBound{0, 0};
+      d.da = max(d.da, s.da);
+      d.db = max(d.db, s.db);
+    }
+  return d;
+}
+
+struct Bounds {
+  int ba, bb;
+  DigitBound d;
+};
+Bounds bounds_of(const ccm_matrix& a, const ccm_matrix& b) {
+  Bounds r;
+  r.ba = width_bound(a.capacity, a.rows * a.cols);
+  r.bb = width_bound(b.capacity, b.rows * b.cols);
+  r.d = digit_bound(r.ba, r.bb);
+  return r;
+}
+
+size_t plane_bytes(uint64_t m, uint64_t k, uint64_t n, int da, int db) {
+  const uint64_t kp = round_up(k, 64);
+  return round_up(2 * (uint64_t)da * m * kp, 256) + round_up(2 * (uint64_t)db * n * kp, 256);
+}
 
 }  // namespace tc
 
-// The tensor path needs both widths bounded by 16 bits (at most 4 digits) and
-// every class sum below 2^24.
 bool matmul_c32(const ccm_matrix& c) { return width_bound(c.capacity, c.rows * c.cols) <= 31; }
 
-bool matmul_tc_supported(const ccm_matrix& a, const ccm_matrix& b) {
+// The product runs on the tensor cores when every width the capacities allow
+// has a split and every sum stays inside int64.
+bool matmul_tc_applies(const ccm_matrix& a, const ccm_matrix& b) {
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  if (!m || !n || !k) return false;
-  const int ba = width_bound(a.capacity, m * k), bb = width_bound(b.capacity, k * n);
-  const int L = tc::digits_for(ba > bb ? ba : bb);
-  if (L < 1 || L > 4) return false;
-  if ((double)k * L * 225.0 >= 16777216.0) return false;
-  if (ba + bb + bitlen_host(k) > 62) return false;
+  if (!m || !n || !k || m >= (1ull << 31) || n >= (1ull << 31) || k >= (1ull << 31)) return false;
+  const tc::Bounds r = tc::bounds_of(a, b);
+  if (!r.d.da || r.ba + r.bb + bitlen_host(k) > 62) return false;
   return tc::encode_fn() != nullptr;
 }
 
-size_t matmul_tc_workspace(const ccm_matrix& a, const ccm_matrix& b) {
-  if (!matmul_tc_supported(a, b)) return 0;
-  const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  const int ba = width_bound(a.capacity, m * k), bb = width_bound(b.capacity, k * n);
-  tc::Plan p = tc::plan_for(m, k, n, tc::digits_for(ba > bb ? ba : bb));
-  return tc::round_up(p.a_bytes, 256) + tc::round_up(p.b_bytes, 256);
+size_t matmul_tc_bytes(const ccm_matrix& a, const ccm_matrix& b) {
+  const tc::Bounds r = tc::bounds_of(a, b);
+  return tc::plane_bytes(a.rows, a.cols, b.cols, r.d.da, r.d.db);
 }
 
-size_t matmul_tc_workspace_upper(uint64_t m, uint64_t k, uint64_t n) {
+size_t matmul_tc_bytes_upper(uint64_t m, uint64_t k, uint64_t n) {
   if (!m || !n || !k) return 0;
-  tc::Plan p = tc::plan_for(m, k, n, 4);
-  return tc::round_up(p.a_bytes, 256) + tc::round_up(p.b_bytes, 256);
+  return tc::plane_bytes(m, k, n, tc::kMaxDigits, tc::kMaxDigits);
 }
 
-template <int L>
-static void launch_mm(const CUtensorMap& ta, const CUtensorMap& tb, const tc::MmArgs& args,
-                      unsigned grid, cudaStream_t st) {
-  constexpr tc::Geo g = tc::geometry(L);
-  const size_t smem = (size_t)g.stages * L * tc::kBK * (tc::kBM + g.bn) + 1024;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(tc::k_mm_tc<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
-  tc::k_mm_tc<L><<<grid, tc::kThreadsP, smem, st>>>(ta, tb, args);
+namespace {
+
+template <int BN, bool kAcc64>
+cudaError_t launch_mm(const CUtensorMap& ta, const CUtensorMap& tb, const tc::MmArgs& args,
+                      unsigned pairs, bool pdl, cudaStream_t st) {
+  using G = tc::Geo<BN, kAcc64>;
+  cudaError_t e = cudaFuncSetAttribute(tc::k_mm<BN, kAcc64>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::kSmem);
+  if (e != cudaSuccess) return e;
+  if (pdl)
+    return ax::launch_pdl(tc::k_mm<BN, kAcc64>, dim3(2 * pairs), dim3(tc::kThreads), G::kSmem, st,
+                          ta, tb, args);
+  tc::k_mm<BN, kAcc64><<<2 * pairs, tc::kThreads, G::kSmem, st>>>(ta, tb, args);
+  return cudaGetLastError();
 }
 
-int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c,
-                  int64_t* c_scratch, void* ws, cudaStream_t st) {
+}  // namespace
+
+int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, void* c_scratch,
+                  void* ws, cudaStream_t st) {
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  const int ba = width_bound(a.capacity, m * k), bb = width_bound(b.capacity, k * n);
-  const int L = tc::digits_for(ba > bb ? ba : bb);
-  tc::Plan p = tc::plan_for(m, k, n, L);
-  uint8_t* pa = (uint8_t*)ws;
-  uint8_t* pb = pa + tc::round_up(p.a_bytes, 256);
+  const tc::Bounds r = tc::bounds_of(a, b);
+  const uint64_t kp = tc::round_up(k, 64);
+  const bool pdl = !profile_armed();
+  __half* pa = (__half*)ws;
+  __half* pb = (__half*)((char*)ws + tc::round_up(2 * (uint64_t)r.d.da * m * kp, 256));
   {
-    const uint64_t quads = p.m_pad * p.k_pad / 4;
-    int g = (int)umin((quads + 255) / 256, (uint64_t)num_sms() * 16);
-    tc::k_limbs_a<<<g, 256, 0, st>>>(c.hdr, a.hdr, a.words, m, k, p.m_pad, p.k_pad, L, pa);
-    const uint64_t tiles = (p.k_pad / 64) * (p.n_pad / 32);
-    int g2 = (int)umin(tiles, (uint64_t)num_sms() * 16);
-    tc::k_limbs_bt<<<g2, 256, 0, st>>>(c.hdr, b.hdr, b.words, k, n, p.n_pad, p.k_pad, L, pb);
-    note_launch(2);
+    tc::PlaneArgs p{c.hdr, a.hdr, b.hdr, a.words, b.words, m, k, n, kp, pa, pb, 0, 0, 0};
+    p.row_runs = (uint32_t)((kp / 8 + 31) / 32);
+    p.blocks_a = (uint32_t)umin((m * p.row_runs + 7) / 8, (uint64_t)num_sms() * 32);
+    p.tiles_k = (uint32_t)(kp / 64);
+    const unsigned grid = (unsigned)(p.blocks_a + p.tiles_k * ((n + 63) / 64));
+    if (pdl)
+      ax::launch_pdl(tc::k_planes, dim3(grid), dim3(256), 0, st, p);
+    else
+      tc::k_planes<<<grid, 256, 0, st>>>(p);
+    note_launch();
   }
-  const tc::Geo g = tc::geometry(L);
+  // 32-bit accumulators when no result can leave int32.  The tile width is the
+  // one with the least loading: the L2 feeds about 46 bytes per clock and SM
+  // (BN = 256: 32 KB per block of k, 90 us at 4096^3; 128: 24 KB, 111 us), so
+  // a wave of tiles costs 128 rows of A and BN / 2 of B per CTA whatever the
+  // MMAs cost.  At 4096^3: 224 columns give exactly 4 waves, 82 us.
+  const bool acc32 = r.ba + r.bb + bitlen_host(k) <= 31;
+  const int sizes32[] = {256, 224, 192, 128, 64}, sizes64[] = {128, 64};
+  const int* sizes = acc32 ? sizes32 : sizes64;
+  const uint64_t tiles_m = (m + tc::kBM - 1) / tc::kBM, pairs = (uint64_t)num_sms() / 2;
+  int bn = 0;
+  double best = 0;
+  for (int i = 0; i < (acc32 ? 5 : 2); ++i) {
+    const uint64_t tiles = tiles_m * ((n + sizes[i] - 1) / sizes[i]);
+    const uint64_t waves = (tiles + pairs - 1) / pairs;
+    const double cost = (double)waves * (256 + sizes[i]);
+    if (!bn || cost < best) {
+      bn = sizes[i];
+      best = cost;
+    }
+  }
+  const uint32_t sub = bn > 128 ? 1 : 2;
   CUtensorMap ta, tb;
-  if (!tc::make_map(&ta, pa, p.k_pad, (uint64_t)L * p.m_pad, tc::kBM) ||
-      !tc::make_map(&tb, pb, p.k_pad, (uint64_t)L * p.n_pad, (uint32_t)g.bn))
+  if (!tc::make_map(&ta, pa, kp, m, r.d.da, 128, sub) ||
+      !tc::make_map(&tb, pb, kp, n, r.d.db, (uint32_t)bn / 2, sub))
     return CCM_E_CUDA;
-  tc::MmArgs args{c.hdr, c_scratch, m, n, (uint32_t)(p.k_pad / tc::kBK), (uint32_t)p.m_pad,
-                  (uint32_t)p.n_pad, (uint32_t)(p.n_pad / g.bn), (uint32_t)(p.m_pad / tc::kBM),
-                  L, matmul_c32(c) ? 1 : 0};
-  // persistent: one CTA per SM (the stages fill its shared memory), or one
-  // per tile when there are fewer tiles
-  const uint64_t tiles = (p.m_pad / tc::kBM) * (p.n_pad / g.bn);
-  const unsigned grid = (unsigned)umin(tiles, (uint64_t)num_sms());
+  tc::MmArgs args{c.hdr, a.hdr, b.hdr, c_scratch, m, n, (uint32_t)((k + tc::kBK - 1) / tc::kBK),
+                  (uint32_t)tiles_m, (uint32_t)((n + bn - 1) / bn), matmul_c32(c) ? 1 : 0};
+  const unsigned grid = (unsigned)umin((uint64_t)args.tiles_m * args.tiles_n, pairs);
+  cudaError_t e = cudaErrorInvalidValue;
   profile_begin(st);
-  switch (L) {
-    case 1: launch_mm<1>(ta, tb, args, grid, st); break;
-    case 2: launch_mm<2>(ta, tb, args, grid, st); break;
-    case 3: launch_mm<3>(ta, tb, args, grid, st); break;
-    default: launch_mm<4>(ta, tb, args, grid, st); break;
+  if (acc32) {
+    switch (bn) {
+      case 256: e = launch_mm<256, false>(ta, tb, args, grid, pdl, st); break;
+      case 224: e = launch_mm<224, false>(ta, tb, args, grid, pdl, st); break;
+      case 192: e = launch_mm<192, false>(ta, tb, args, grid, pdl, st); break;
+      case 128: e = launch_mm<128, false>(ta, tb, args, grid, pdl, st); break;
+      default: e = launch_mm<64, false>(ta, tb, args, grid, pdl, st); break;
+    }
+  } else {
+    switch (bn) {
+      case 128: e = launch_mm<128, true>(ta, tb, args, grid, pdl, st); break;
+      default: e = launch_mm<64, true>(ta, tb, args, grid, pdl, st); break;
+    }
   }
   profile_end(st);
   note_launch();
-  return CCM_OK;
+  return e == cudaSuccess ? CCM_OK : CCM_E_CUDA;
 }
 
 }  // namespace ccm
