@@ -10,10 +10,8 @@
 namespace ccm {
 namespace ax {
 
-// A bounded wait suspends for up to kSuspendNs at a time (the hint of
-// try_wait; without it a waiting warp polls and its polls hold up the shared
-// memory accesses of the others), and gives up after about two seconds.
-constexpr uint32_t kSuspendNs = 1000000;
+// Polls of one bounded wait before it gives up; with the globaltimer check
+// below a wait never lasts more than about two seconds.
 constexpr uint32_t kSpinLimit = 1u << 26;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -42,9 +40,37 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 }
 
 // Bounded wait for the phase of parity `parity` to complete: false after
-// about two seconds (or kSpinLimit polls), never an endless spin.  The clock
-// is read only after a failed poll.
+// about two seconds (or kSpinLimit polls), never an endless spin.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  const uint32_t addr = smem_u32(bar);
+  uint64_t t0 = 0;
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 1023) == 0) {
+      const uint64_t now = globaltimer_ns();
+      if (it == 0)
+        t0 = now;
+      else if (now - t0 > 2000000000ull)
+        return false;
+    }
+  }
+  return false;
+}
+
+// The same for a warp that waits long beside others that are busy: suspended
+// for up to a millisecond at a time (the hint of try_wait), where the polls of
+// mbar_wait would hold up the others' shared memory accesses (the matmul's
+// issue loop: 554 -> 593 TOPS).  The per-warp rings keep mbar_wait: their waits
+// are short, and the suspended form cost them 2 %.
+__device__ __forceinline__ bool mbar_wait_suspended(uint64_t* bar, uint32_t parity) {
   const uint32_t addr = smem_u32(bar);
   uint64_t t0 = 0;
   for (uint32_t it = 0; it < kSpinLimit; ++it) {
@@ -54,7 +80,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
         "selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(addr), "r"(parity), "r"(kSuspendNs)
+        : "r"(addr), "r"(parity), "r"(1000000u)
         : "memory");
     if (done) return true;
     const uint64_t now = globaltimer_ns();

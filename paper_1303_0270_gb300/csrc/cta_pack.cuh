@@ -1,8 +1,8 @@
-// cta_pack.cuh -- a short vector of int64 values (up to 16,384) packed by a
+// cta_pack.cuh -- a short vector of int64 values (up to 65,536) packed by a
 // small grid in one launch: every CTA reads all the values for the width
 // statistics (a few hundred KB of L2 reads at most), stages only its own
 // groups of 32 fields in shared memory and packs them; CTA 0 writes the
-// header and the pad words.  No CTA waits for another (k_mv_ypack's y,
+// header and the pad words.  No CTA waits for another (k_pack_vec's y,
 // k_pack_small's small dense input).
 #pragma once
 

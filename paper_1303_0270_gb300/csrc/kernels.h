@@ -40,7 +40,7 @@ void run_scale(const ccm_matrix& a, int64_t s, const ccm_matrix& c, void* ws, si
 // Packs an int64 result held in scratch; `stats_done` when the producing
 // kernel has already merged the width statistics into out's header.
 void run_pack_scratch(const int64_t* vals, const ccm_matrix& out, cudaStream_t st,
-                      bool stats_done = false);
+                      bool stats_done = false, bool pdl = false);
 // The same from an int32 scratch whose width statistics the producing kernel
 // has already merged into out's header.
 void run_pack_scratch32(const int32_t* vals, const ccm_matrix& out, cudaStream_t st);
@@ -59,6 +59,12 @@ bool stream_applies(uint64_t m, uint64_t n, int bmax_a, int bmax_x);
 void run_stream(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, void* ws,
                 cudaStream_t st);
 }  // namespace mvs
+// The matvec of rows that begin anywhere in a word (matvec_ragged.cu).
+namespace mvr {
+bool ragged_applies(uint64_t m, uint64_t n, int bmax_a, int bmax_x);
+void run_ragged(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, void* ximg,
+                int64_t* yv, bool fresh, cudaStream_t st);
+}  // namespace mvr
 size_t matvec2_workspace(uint64_t m, uint64_t n1, uint64_t n2);
 void run_matvec2(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& b,
                  const ccm_matrix& z, const ccm_matrix& y, void* ws, cudaStream_t st);

@@ -53,7 +53,6 @@ namespace ccm {
 namespace tc {
 
 using ax::mbar_init;
-using ax::mbar_wait;
 using ax::smem_u32;
 
 constexpr int kBM = 256;          // rows of C per CTA pair (128 per CTA)
@@ -554,7 +553,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int l = p / sp.db, q = p % sp.db;
         if (abort_s) ok = false;
         for (uint32_t kb = 0; kb < nk && ok; ++kb) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], parity))) {
+          if (!__all_sync(0xffffffffu, ax::mbar_wait_suspended(&empty_bar[s], parity))) {
             ok = false;
             break;
           }
@@ -575,7 +574,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (lane == 0) issued_s = issued;
     // the leader's commits still on their way to this CTA's barriers
     for (uint32_t x = issued > (uint32_t)S ? issued - S : 0; x < issued && ok; ++x)
-      ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[x % S], (x / S) & 1));
+      ok = __all_sync(0xffffffffu, ax::mbar_wait_suspended(&empty_bar[x % S], (x / S) & 1));
     if (!ok) abort_s = 1;
   } else if (warp == 1) {
     if (rank == 0) {
@@ -589,7 +588,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           for (uint32_t k0 = 0; k0 < nk && ok; k0 += run, ++f) {
             const uint32_t buf = f % G::kBufs;
             if (abort_s || !__all_sync(0xffffffffu,
-                                       mbar_wait(&acc_empty[buf], ((f / G::kBufs) & 1) ^ 1))) {
+                                       ax::mbar_wait_suspended(&acc_empty[buf], ((f / G::kBufs) & 1) ^ 1))) {
               ok = false;
               break;
             }
@@ -597,7 +596,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const uint32_t acc = tmem0 + buf * G::kBufCols;
             const uint32_t k1 = k0 + run < nk ? k0 + run : nk;
             for (uint32_t kb = k0; kb < k1; ++kb) {
-              if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], parity))) {
+              if (!__all_sync(0xffffffffu, ax::mbar_wait_suspended(&full_bar[s], parity))) {
                 ok = false;
                 break;
               }
@@ -645,7 +644,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (uint32_t k0 = 0; k0 < nk; k0 += run, ++f) {
           const uint32_t buf = f % G::kBufs;
           // (one decision for the whole warp: the tensor-memory loads are warp-wide)
-          if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (f / G::kBufs) & 1)) ||
+          if (!__all_sync(0xffffffffu, ax::mbar_wait_suspended(&acc_full[buf], (f / G::kBufs) & 1)) ||
               __any_sync(0xffffffffu, abort_s != 0)) {
             ok = false;
             break;
@@ -706,7 +705,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (rank == 0) {
       const uint32_t issued = issued_s;
       for (uint32_t g = issued > (uint32_t)S ? issued - S : 0; g < issued; ++g)
-        if (!mbar_wait(&full_bar[g % S], (g / S) & 1)) break;
+        if (!ax::mbar_wait_suspended(&full_bar[g % S], (g / S) & 1)) break;
     }
     if (abort_s) set_status(args.out, CCM_E_TIMEOUT);
   }

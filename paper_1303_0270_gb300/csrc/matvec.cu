@@ -4,14 +4,13 @@
 // partial sum below 2^63, in 128-bit integers otherwise; y is then re-packed
 // at its own width by the pack engine.
 //
-// Launch sequence on the stream:
-//   k_init          validate A (m x n) and x (n x 1), clear y's header and
-//                   the int64 y scratch
-//   k_matvec_fast   when cols % 128 == 0 and the buffers bound both widths
-//                   by 31/32 bits (see matvec_fast.cuh); otherwise
-//     k_decode_vec  x -> int64 scratch, and
-//     k_matvec_rows one warp per row, fields decoded from A's words
-//   k_stats, k_pack y scratch -> packed y
+// run_matvec chooses among the streaming kernel (matvec_stream.cu), the segment
+// kernel (matvec_ragged.cu) and, on an int64 y scratch cleared by k_init, the
+// row and column-slab kernels (matvec_fast.cuh) and, where the widths need
+// it, the generic kernel:
+//   k_decode_vec  x -> int64 scratch, and
+//   k_matvec_rows one warp per row, fields decoded from A's words
+// y is then packed by run_pack_scratch.
 //
 // The host cannot see the widths (they live in device headers), but a
 // buffer of `capacity` words can only hold a matrix of width
@@ -285,6 +284,10 @@ void matvec_term(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, 
       return;
     }
   }
+  if (mvr::ragged_applies(m, n, bmax_a, bmax_x) && bmax_a + bmax_x + bitlen_host(n) <= budget) {
+    mvr::run_ragged(a, x, y, xs, yv, /*fresh=*/false, st);
+    return;
+  }
   // generic: x decoded to int64, one warp per row, 128-bit sums when needed
   int g = (int)umin((n + 255) / 256, (uint64_t)num_sms() * 4);
   k_decode_vec<<<g, 256, 0, st>>>(y.hdr, x.hdr, x.words, n, xs);
@@ -319,14 +322,34 @@ InitArgs matvec_init(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix&
 void run_matvec(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, void* ws,
                 cudaStream_t st) {
   const uint64_t n_a = a.rows * a.cols;
-  if (mvs::stream_applies(a.rows, a.cols, width_bound(a.capacity, n_a),
-                          width_bound(x.capacity, a.cols))) {
+  const int bmax_a = width_bound(a.capacity, n_a), bmax_x = width_bound(x.capacity, a.cols);
+  const bool ragged = mvr::ragged_applies(a.rows, a.cols, bmax_a, bmax_x) &&
+                      bmax_a + bmax_x + bitlen_host(a.cols) <= 63;
+  // Rows of whole 128-column chunks.  b <= 8: the streaming kernel's byte lanes
+  // (8192^2 at 5 bits 22 us, the segment kernel 28), but x of 9 to 14 bits,
+  // which it takes as int32, goes to the segment kernel's byte digits (3 x 12
+  // bits 25 us against 29).  Wider: the segment kernel (8192^2 at 12 / 20 / 28
+  // bits 34 / 47 / 50 us, the row kernel 38 / 50 / 74), except large A at 16
+  // and 24 bits, whose segments share banks (48 and 65 us against 43 and 54),
+  // rows too long for x in L1 (3000 x 262144 at 5 bits 163 against 131 us) and
+  // x past the byte digits.
+  const bool chunks = a.cols % mvf::kKC == 0;
+  const bool byte_digits = bmax_x <= 14;
+  if (!(ragged && bmax_x > 8 && byte_digits) &&
+      mvs::stream_applies(a.rows, a.cols, bmax_a, bmax_x)) {
     mvs::run_stream(a, x, y, ws, st);
     return;
   }
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
   int64_t* xs = (int64_t*)ws;
   int64_t* yv = (int64_t*)((char*)ws + up(a.cols * sizeof(int64_t)));
+  const bool banks = (bmax_a == 16 || bmax_a == 24) && n_a >= (1ull << 24);
+  if (ragged && !(chunks && (!byte_digits || a.cols > 65536 || banks))) {
+    const bool pdl = !profile_armed();
+    mvr::run_ragged(a, x, y, xs, yv, /*fresh=*/true, st);
+    run_pack_scratch(yv, y, st, /*stats_done=*/false, pdl);
+    return;
+  }
   launch_init(matvec_init(a, x, y, yv), st);
   matvec_term(a, x, y, xs, yv, 63, st);
   run_pack_scratch(yv, y, st);

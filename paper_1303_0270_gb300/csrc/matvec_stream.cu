@@ -1,12 +1,11 @@
 // matvec_stream.cu -- the launch chain of the streaming matvec (see
-// matvec_stream.cuh): k_mv_init, k_mv, k_mv_ypack, the last two started by
-// programmatic dependent launch.
+// matvec_stream.cuh): k_mv_init, k_mv and the pack of y, the last two started
+// by programmatic dependent launch.
 #include <map>
 #include <mutex>
 
 #include "kernels.h"
 #include "matvec_stream.cuh"
-#include "cta_pack.cuh"
 #include "pack_engine.cuh"
 
 namespace ccm {
@@ -68,43 +67,12 @@ __global__ void __launch_bounds__(kInitThreads) k_mv_init(Args a) {
   }
 }
 
-// y's width (statistics of the int64 sums), header, and y packed at that
-// width, by vec_pack_ctas(m) CTAs: each reads all the sums for the
-// statistics and packs its own 16 groups of 32 fields (cta_pack.cuh); CTA 0
-// writes the header.
-__global__ void __launch_bounds__(kVecThreads) k_mv_ypack(ccm_header* out, uint32_t* words,
-                                                          uint64_t capacity,
-                                                          const int64_t* __restrict__ y,
-                                                          uint64_t m) {
-  __shared__ VecPackSmem sm;
-  ax::grid_dep_wait();  // every sum of k_mv is in place
-  if (out->status != CCM_OK) return;
-  const uint32_t mm = (uint32_t)m;  // <= kYSmallRows
-  const uint32_t g0 = blockIdx.x * kVecGroupsPerCta;
-  uint64_t orv;
-  uint32_t neg;
-  vec_stats_stage([&](uint32_t i) { return y[i]; }, mm, g0, sm, orv, neg);
-  const int b = width_from_stats(orv, neg);
-  const uint64_t nw = words_for(m, b), dw = data_words(m, b);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    out->stat_or = orv;
-    out->stat_neg = neg;
-    out->width = b;
-    out->is_signed = neg ? 1 : 0;
-    out->nwords = nw;
-    out->magic = CCM_MAGIC;
-    if (nw > capacity) out->status = CCM_E_CAPACITY;
-  }
-  if (nw > capacity) return;
-  vec_pack_groups(sm, mm, g0, b, words, dw, nw);
-}
-
 std::mutex g_attr_mutex;
 int g_attr_dev = -1;
 std::map<uint64_t, std::pair<int, int>> g_plans;  // (device, widths, path) -> (ring depth, CTAs per SM)
 size_t g_dyn_max = 0;  // dynamic shared memory k_mv may use (opt-in minus its static share)
 
-// Opt-in shared memory for k_mv and k_mv_ypack on the current device (once):
+// Opt-in shared memory for k_mv on the current device (once):
 // the largest dynamic size is the opt-in limit minus the kernel's static
 // shared memory.
 size_t set_attrs() {
@@ -207,17 +175,7 @@ void run_stream(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, v
     ax::launch_pdl(kmv, dim3((unsigned)grid), dim3(kWarps * 32), smem, st, args);
   profile_end(st);
   note_launch();
-  if (m <= kYSmallRows) {
-    const uint32_t g = vec_pack_ctas(m);
-    if (plain)
-      k_mv_ypack<<<g, kVecThreads, 0, st>>>(y.hdr, y.words, y.capacity, (const int64_t*)yv, m);
-    else
-      ax::launch_pdl(k_mv_ypack, dim3(g), dim3(kVecThreads), 0, st, y.hdr, y.words,
-                     y.capacity, (const int64_t*)yv, m);
-    note_launch();
-  } else {
-    run_pack_scratch(yv, y, st);
-  }
+  run_pack_scratch(yv, y, st, /*stats_done=*/false, /*pdl=*/!plain);
 }
 
 }  // namespace mvs

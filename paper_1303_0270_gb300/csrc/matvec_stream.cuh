@@ -1,14 +1,13 @@
 // matvec_stream.cuh -- y = A x for row-aligned A (cols a multiple of 128)
 // whose fields have at most 8 bits: the streaming kernel of ccm_matvec.
 //
-// One call is three launches chained by programmatic dependent launch, so
+// One call is launches chained by programmatic dependent launch, so
 // each starts while the previous one finishes:
 //   k_mv_init   validates A and x, clears y's header and the int64 y sums,
 //               and decodes x once into an image in the workspace;
 //   k_mv        streams A: it issues its first copies of A before it waits
 //               for k_mv_init (A does not depend on it);
-//   k_mv_ypack  y's width statistics and y packed at that width, by one CTA
-//               (y of up to kYSmallRows rows; larger y use the pack engine).
+//   y's width statistics and y packed at that width (run_pack_scratch).
 //
 // k_mv: the packed A is cut into warp-stages of up to 32 consecutive
 // 128-field chunks of one row (a chunk is 16*b contiguous bytes, 16-byte
@@ -45,7 +44,6 @@ using mvf::kKC;
 constexpr int kChunks = 32;     // chunks of a warp-stage (one per lane)
 constexpr int kWarps = 8;       // warps of a CTA
 constexpr int kMaxSlots = 6;    // ring slots of a warp
-constexpr uint64_t kYSmallRows = 16384;
 
 // Shared bytes of one ring slot (one warp-stage, chunks back to back) for width b.
 __host__ __device__ constexpr uint32_t slot_bytes(int b) { return kChunks * 16u * (uint32_t)b; }

@@ -506,11 +506,59 @@ void run_pack_scratch32(const int32_t* vals, const ccm_matrix& out, cudaStream_t
   launch_pack(ProdDenseI32{vals}, out.hdr, out.words, out.capacity, n, st);
 }
 
+// Width, header and words of a vector of int64 values (y of a matvec) in one
+// launch of vec_pack_ctas(n) CTAs: each reads all the values for the
+// statistics (from L2) and packs its own 16 groups of 32 fields (cta_pack.cuh);
+// CTA 0 writes the header.
+__global__ void __launch_bounds__(kVecThreads) k_pack_vec(ccm_header* out, uint32_t* words,
+                                                          uint64_t capacity,
+                                                          const int64_t* __restrict__ y,
+                                                          uint64_t m) {
+  __shared__ VecPackSmem sm;
+  ax::grid_dep_wait();  // every sum is in place
+  if (out->status != CCM_OK) return;
+  const uint32_t mm = (uint32_t)m;  // <= kVecMax
+  const uint32_t g0 = blockIdx.x * kVecGroupsPerCta;
+  uint64_t orv;
+  uint32_t neg;
+  vec_stats_stage([&](uint32_t i) { return y[i]; }, mm, g0, sm, orv, neg);
+  const int b = width_from_stats(orv, neg);
+  const uint64_t nw = words_for(m, b), dw = data_words(m, b);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    out->stat_or = orv;
+    out->stat_neg = neg;
+    out->width = b;
+    out->is_signed = neg ? 1 : 0;
+    out->nwords = nw;
+    out->magic = CCM_MAGIC;
+    if (nw > capacity) out->status = CCM_E_CAPACITY;
+  }
+  if (nw > capacity) return;
+  vec_pack_groups(sm, mm, g0, b, words, dw, nw);
+}
+
+// Longest vector of the one-launch pack: every CTA reads all of it (512 KB at
+// this length, a few us), which up to here beats a statistics pass and a pack
+// pass (20,011 sums: 16 us).
+constexpr uint64_t kVecMax = 65536;
+
 // Pack an int64 result held in device scratch (matvec / matmul epilogue).
+// `pdl`: may start while the kernel that writes `vals` still runs (it waits
+// for it).
 void run_pack_scratch(const int64_t* vals, const ccm_matrix& out, cudaStream_t st,
-                      bool stats_done) {
+                      bool stats_done, bool pdl) {
   ProdDenseI64 p{vals};
   uint64_t n = out.rows * out.cols;
+  if (n && n <= kVecMax && !stats_done) {
+    const uint32_t g = vec_pack_ctas(n);
+    if (pdl)
+      ax::launch_pdl(k_pack_vec, dim3(g), dim3(kVecThreads), 0, st, out.hdr, out.words,
+                     out.capacity, vals, n);
+    else
+      k_pack_vec<<<g, kVecThreads, 0, st>>>(out.hdr, out.words, out.capacity, vals, n);
+    note_launch();
+    return;
+  }
   const int cls = ew_class(width_bound(out.capacity, n));
   if (cls && n) {
     if (!stats_done) launch_stats(p, out.hdr, n, st);
