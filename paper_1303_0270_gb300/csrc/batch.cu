@@ -5,47 +5,28 @@
 // fields; segments are numbered row-major within a matrix, and a work unit is
 // a run of consecutive segments of one matrix (the plan's unit list).  Every
 // warp of the persistent kernel takes units from an atomic ticket of its own
-// (no CTA barrier: the warps of a CTA are independent) and streams them
-// through a ring of D slots in shared memory.  A stage is 32 P consecutive
-// segments of one unit (P segments per lane, about `stage_bytes` bytes of A
-// whatever the width); its word range is brought in by one 1-D
-// cp.async.bulk completing on the slot's mbarrier, so D - 1 stages are in
-// flight while one is decoded.  The warp fetches its next unit's ticket one
-// unit ahead, so the ring runs on across unit and matrix boundaries.
-//
-// Lane l of a stage's sub-step p decodes segment 32 p + l: it reads the b + 1
-// words that cover the segment from the slot and funnel-shifts them once to
-// the segment's first bit (a segment starts at an arbitrary bit).  Fast
-// path (b <= 24 and x of at most 8 signed bits, or 7 unsigned): x is decoded
-// once into bytes and the segment's dot product runs on the integer dot
-// units -- four fields spread into the bytes of a register per dp4a
-// (b <= 8), two into the halves per dp2a (b <= 16), signed fields in offset
-// binary corrected by 2^(b-1) times the segment's sum of x; b = 17..24 takes
-// one 32 x 32 -> 64 multiply-add per field.  Other entries take the general
-// path (int32 x image, one 64-bit multiply-add per field).  Lanes hold
-// consecutive segments, so the rows of a sub-step are runs of lanes: one row
-// is summed with two redux.sync, several with a segmented shuffle reduction;
-// each row's partial sum is added to the int64 y scratch with one atomic.
+// (no CTA barrier: the warps of a CTA are independent) and runs each through
+// its ring of D slots with the width-specialised segment code
+// (segment_range.cuh).  The next unit's ticket, record and matrix are fetched
+// while the first copies of the unit at hand are under way, so a unit begins
+// with its copies.
 //
 // The tickets hand out the units in the order of their matrices' codes
-// (width, sign, path): a one-CTA kernel after the initialisation sorts them
-// by counting.  So at any time the warps of an SM decode one or two widths,
-// and the code of one width-specialised decode stays in the instruction
-// cache (with units in plan order, the warps of an SM ran up to 24 different
-// decode bodies at once and mostly waited for instruction fetch).
+// (width, sign, form of x): after the initialisation a kernel sorts them by
+// counting.  So at any time the warps of an SM decode one or two widths, and
+// the code of one width-specialised decode stays in the instruction cache.
 //
 // The warp that completes the last unit of a matrix (per-matrix counter)
 // re-packs that matrix's y at its exact width (width rule of Eq. 1 with the
-// two's complement reading) and writes y's header.  The whole batch is one
-// launch after a small initialisation kernel, and both can be captured in a
-// CUDA graph.
+// two's complement reading) and writes y's header.  The launches can be
+// captured in a CUDA graph.
 #include <cstring>
 #include <vector>
 
 #include "async_copy.cuh"
 #include "ccm_device.cuh"
 #include "kernels.h"
-#include "segment_dot.cuh"
+#include "segment_range.cuh"
 
 namespace ccm {
 namespace bt {
@@ -55,32 +36,7 @@ using namespace seg;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCols = 8192;       // x of at most 8192 entries per matrix
-constexpr int kMaxSlots = 4;         // ring depth limit
-constexpr int kMaxLaneSegs = 8;      // segments per lane in one stage
 constexpr uint32_t kDefaultStageBytes = 3072;
-constexpr int kFastMaxWidth = 24;    // widest A on the byte-dot path
-
-// Segments per lane of one stage at width b: about stage_bytes of A per
-// warp stage (a sub-step of 32 segments holds 128 b bytes).
-__host__ __device__ inline uint32_t lane_segments(uint32_t stage_bytes, int b) {
-  const uint32_t p = stage_bytes / (128u * (uint32_t)b);
-  return p < 1 ? 1u : (p > (uint32_t)kMaxLaneSegs ? (uint32_t)kMaxLaneSegs : p);
-}
-
-// Bytes of one ring slot: the largest stage at any width up to bmax (at most
-// 128 P b bytes of fields) plus what the reads around it need.  The copy
-// starts up to 12 bytes before the stage's first bit (16-byte rounding) and
-// a lane reads b + 1 words from its segment's first word, also when the
-// segment is the short last one of a row: the highest word read is at most
-// 32 P b + 4 + b words into the slot.
-__host__ __device__ inline uint32_t slot_bytes(uint32_t stage_bytes, int bmax) {
-  uint32_t m = 0;
-  for (int b = 1; b <= bmax; ++b) {
-    const uint32_t v = lane_segments(stage_bytes, b) * 128u * (uint32_t)b + 4u * (uint32_t)b;
-    m = v > m ? v : m;
-  }
-  return (m + 64u + 127u) & ~127u;
-}
 
 struct Mat {
   const ccm_header* ha;
@@ -108,10 +64,14 @@ struct Unit {
 
 // Per-matrix run-time code, written by k_batch_init from the headers: 0 for
 // an entry that is skipped (its y header holds the error), else
-// width | sign << 7 | fast path << 8 | segments per lane << 9.
-constexpr uint32_t kCodeSign = 1u << 7, kCodeFast = 1u << 8;
+// width | sign << 7 | (2 - form of x) << 8: a field per lane, the slowest form,
+// sorts first, so that the last units are not the longest.
+__device__ __forceinline__ uint32_t make_code(int b, int sgn, XMode mode) {
+  return (uint32_t)b | (sgn ? 1u << 7 : 0u) | ((2u - (uint32_t)mode) << 8);
+}
 __device__ __forceinline__ int code_width(uint32_t c) { return (int)(c & 127u); }
-__device__ __forceinline__ uint32_t code_lane_segs(uint32_t c) { return (c >> 9) & 15u; }
+__device__ __forceinline__ bool code_signed(uint32_t c) { return (c >> 7) & 1u; }
+__device__ __forceinline__ XMode code_mode(uint32_t c) { return (XMode)(2u - (c >> 8)); }
 
 struct Args {
   const Mat* mats;
@@ -122,7 +82,7 @@ struct Args {
   uint32_t* done;       // per-matrix completed units
   uint32_t* codes;      // per-matrix run-time code
   uint32_t* order;      // unit indices in code order; order[nunits] = their count
-  int* ximage;          // decoded x of every matrix (Mat::x_off)
+  int* ximage;          // x image of every matrix (Mat::x_off)
   uint32_t slot_bytes;  // bytes of one ring slot
   uint32_t stage_bytes; // target bytes of A per stage
   uint32_t slots;       // ring depth D (2..4)
@@ -133,18 +93,22 @@ struct Args {
 // Initialisation: validate inputs, write y headers and codes, clear counters
 // and the y scratch, decode x into its image.
 // ---------------------------------------------------------------------------
-__global__ void k_batch_init(Args a) {
-  __shared__ int s_st;
-  __shared__ uint32_t s_code;
+constexpr int kInitThreads = 128;
+__global__ void __launch_bounds__(kInitThreads) k_batch_init(const __grid_constant__ Args a) {
   const uint32_t i = blockIdx.x;  // one block per matrix
   const Mat& M = a.mats[i];
+  // (every thread reads the headers: one round trip, no barrier)
+  const HeaderView ha = load_header(M.ha), hx = load_header(M.hx);
+  int st = check_header(ha, M.m, M.n, M.a_cap);
+  if (st == CCM_OK) st = check_header(hx, M.n, 1, M.x_cap);
+  // widths the kernel handles, and sums that provably fit int64
+  if (st == CCM_OK && (ha.width > (int)a.bmax || hx.width > kMaxX ||
+                       ha.width + hx.width + bitlen64(M.n) > 63))
+    st = CCM_E_WIDTH;
+  const uint32_t nsr = M.nseg_row;
+  const int bx = hx.width, sx = hx.is_signed;
+  const XMode mode = x_mode(ha.width, bx, sx, nsr);
   if (threadIdx.x == 0) {
-    int st = check_input(M.ha, M.m, M.n, M.a_cap);
-    if (st == CCM_OK) st = check_input(M.hx, M.n, 1, M.x_cap);
-    // widths the kernel handles, and sums that provably fit int64
-    if (st == CCM_OK && (M.ha->width > (int)a.bmax || M.hx->width > 31 ||
-                         M.ha->width + M.hx->width + bitlen64(M.n) > 63))
-      st = CCM_E_WIDTH;
     ccm_header* y = M.hy;
     y->magic = CCM_MAGIC;
     y->width = 0;
@@ -157,68 +121,53 @@ __global__ void k_batch_init(Args a) {
     y->stat_neg = 0;
     a.done[i] = 0;
     if (i == 0) *a.ticket = 0;
-    uint32_t code = 0;
-    if (st == CCM_OK) {
-      const int b = M.ha->width, bx = M.hx->width, sx = M.hx->is_signed;
-      const bool fast = b <= kFastMaxWidth && (sx ? bx <= 8 : bx <= 7);
-      code = (uint32_t)b | (M.ha->is_signed ? kCodeSign : 0u) | (fast ? kCodeFast : 0u) |
-             (lane_segments(a.stage_bytes, b) << 9);
-    }
-    a.codes[i] = code;
-    s_st = st;
-    s_code = code;
+    a.codes[i] = st == CCM_OK ? make_code(ha.width, ha.is_signed, mode) : 0;
   }
-  for (uint32_t r = threadIdx.x; r < M.m; r += blockDim.x) a.yscratch[M.y_off + r] = 0;
-  __syncthreads();
-  if (s_st != CCM_OK) return;
-  const int bx = M.hx->width, sx = M.hx->is_signed;
-  const uint32_t nsr = M.nseg_row;
-  int* xi = a.ximage + M.x_off;
-  if (s_code & kCodeFast) {
-    // bytes: [half][segment][16], half h holding image bytes 16 h .. 16 h + 15;
-    // then the per-segment sums of x (int).  A warp covers whole segments.
-    const int b = code_width(s_code);
-    int8_t* xb = reinterpret_cast<int8_t*>(xi);
-    int* xsum = xi + 8 * nsr;
-    for (uint32_t j = threadIdx.x; j < nsr * 32; j += blockDim.x) {
-      const uint32_t seg = j / 32, f = j % 32;
-      const int v = j < M.n ? (int)decode_field(M.wx, j, bx, sx) : 0;
-      const uint32_t pos = xbyte_pos(f, b);
-      xb[(pos / 16) * 16 * nsr + 16 * seg + pos % 16] = (int8_t)v;
-      const int s = __reduce_add_sync(0xffffffffu, v);
-      if (f == 0) xsum[seg] = s;
-    }
-  } else {
-    // int32, layout [f/4][segment][f%4], zero past n
-    for (uint32_t j = threadIdx.x; j < nsr * 32; j += blockDim.x) {
-      const uint32_t seg = j / 32, f = j % 32;
-      xi[((f / 4) * nsr + seg) * 4 + (f % 4)] = j < M.n ? (int)decode_field(M.wx, j, bx, sx) : 0;
-    }
+  for (uint32_t r = threadIdx.x; r < M.m; r += kInitThreads) a.yscratch[M.y_off + r] = 0;
+  if (st != CCM_OK) return;
+  uint8_t* img = reinterpret_cast<uint8_t*>(a.ximage + M.x_off);
+  const uint32_t lane = threadIdx.x % 32;
+#pragma unroll 2
+  for (uint32_t s = threadIdx.x / 32; s < nsr; s += kInitThreads / 32) {
+    const uint32_t j = 32 * s + lane;
+    write_x(img, nsr, s, lane, j < M.n ? (int)decode_field(M.wx, j, bx, sx) : 0, ha.width, mode);
   }
 }
 
 // ---------------------------------------------------------------------------
-// Unit order: a counting sort of the valid entries' units by code, one CTA.
+// Unit order: a counting sort of the valid entries' units by code.  Each CTA
+// counts all the entries (their codes and unit counts are a few KB) and those
+// before its own slice, so it knows where its slice's units of every code go
+// without waiting for another CTA; then a warp writes an entry's units.  (By
+// one CTA, with one thread per entry: 105 us for 10,000 matrices.)
 // ---------------------------------------------------------------------------
-constexpr int kOrderThreads = 1024;
-constexpr int kCodes = 512;  // codes & 0x1ff
+constexpr int kOrderThreads = 512;
+constexpr int kCodes = 1024;  // codes: width, sign, form of x
 
-__global__ void __launch_bounds__(kOrderThreads) k_batch_order(Args a) {
-  __shared__ uint32_t s_cnt[kCodes];
-  for (int c = threadIdx.x; c < kCodes; c += blockDim.x) s_cnt[c] = 0;
+__global__ void __launch_bounds__(kOrderThreads) k_batch_order(const __grid_constant__ Args a) {
+  __shared__ uint32_t s_cnt[kCodes];   // units of every code, then where they begin
+  __shared__ uint32_t s_mine[kCodes];  // units of the entries before this slice
+  __shared__ uint32_t s_warp[kOrderThreads / 32];
+  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+  for (int c = tid; c < kCodes; c += kOrderThreads) s_cnt[c] = s_mine[c] = 0;
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < a.nmats; i += blockDim.x) {
-    const uint32_t code = a.codes[i];
-    if (code) atomicAdd(&s_cnt[code & (kCodes - 1)], a.mats[i].units);
+  const uint32_t i0 = (uint32_t)((uint64_t)a.nmats * blockIdx.x / gridDim.x);
+  const uint32_t i1 = (uint32_t)((uint64_t)a.nmats * (blockIdx.x + 1) / gridDim.x);
+#pragma unroll 4
+  for (uint32_t i = tid; i < a.nmats; i += kOrderThreads) {
+    const uint32_t code = a.codes[i], units = a.mats[i].units;
+    if (!code) continue;
+    atomicAdd(&s_cnt[code & (kCodes - 1)], units);
+    if (i < i0) atomicAdd(&s_mine[code & (kCodes - 1)], units);
   }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    // exclusive scan of the 512 counts by one warp, 16 per lane
-    const int lane = threadIdx.x;
-    uint32_t v[kCodes / 32], sum = 0;
+  {
+    // exclusive scan of the counts, kCodes / kOrderThreads per thread
+    constexpr int kPer = kCodes / kOrderThreads;
+    uint32_t v[kPer], sum = 0;
 #pragma unroll
-    for (int k = 0; k < kCodes / 32; ++k) {
-      v[k] = s_cnt[lane * (kCodes / 32) + k];
+    for (int k = 0; k < kPer; ++k) {
+      v[k] = s_cnt[tid * kPer + k];
       sum += v[k];
     }
     uint32_t incl = sum;
@@ -227,125 +176,27 @@ __global__ void __launch_bounds__(kOrderThreads) k_batch_order(Args a) {
       const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
       if (lane >= d) incl += o;
     }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
     uint32_t run = incl - sum;
+    for (int w = 0; w < warp; ++w) run += s_warp[w];
+    if (blockIdx.x == 0 && tid == kOrderThreads - 1) a.order[a.nunits] = run + sum;  // to hand out
 #pragma unroll
-    for (int k = 0; k < kCodes / 32; ++k) {
-      s_cnt[lane * (kCodes / 32) + k] = run;
+    for (int k = 0; k < kPer; ++k) {
+      s_mine[tid * kPer + k] += run;
       run += v[k];
     }
-    if (lane == 31) a.order[a.nunits] = incl;  // units to hand out
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < a.nmats; i += blockDim.x) {
+  for (uint32_t i = i0 + warp; i < i1; i += kOrderThreads / 32) {
     const uint32_t code = a.codes[i];
     if (!code) continue;
-    const Mat& M = a.mats[i];
-    const uint32_t at = atomicAdd(&s_cnt[code & (kCodes - 1)], M.units);
-    for (uint32_t k = 0; k < M.units; ++k) a.order[at + k] = M.unit0 + k;
+    const uint32_t units = a.mats[i].units, unit0 = a.mats[i].unit0;
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(&s_mine[code & (kCodes - 1)], units);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (uint32_t k = lane; k < units; k += 32) a.order[at + k] = unit0 + k;
   }
-}
-
-// ---------------------------------------------------------------------------
-// Dot products of one segment on the general path
-// ---------------------------------------------------------------------------
-// General path: x int32 in the [f/4][segment][f%4] image (xv = image + s).
-template <int B, bool SGN>
-__device__ __forceinline__ int64_t seg_dot_gen(const uint32_t (&f)[B + 1], const int4* __restrict__ xv,
-                                               uint32_t nsr) {
-  long long acc = 0;
-#pragma unroll
-  for (int f4 = 0; f4 < 8; ++f4) {
-    const int4 xq = __ldg(xv + f4 * nsr);
-    const int xa[4] = {xq.x, xq.y, xq.z, xq.w};
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-      const int e = 4 * f4 + qq;
-      const int b0 = e * B, wi = b0 >> 5, sh = b0 & 31;
-      const uint32_t t = (sh + B <= 32) ? (f[wi] >> sh) : __funnelshift_r(f[wi], f[wi + 1], sh);
-      if constexpr (B == 32 && !SGN) {
-        acc += (long long)t * xa[qq];
-      } else {
-        int v;
-        if constexpr (B == 32)
-          v = (int)t;
-        else if constexpr (SGN)
-          v = (int)(t << (32 - B)) >> (32 - B);
-        else
-          v = (int)(t & low_bits(B));
-        acc += (long long)v * (long long)xa[qq];
-      }
-    }
-  }
-  return acc;
-}
-
-// General path: adds each lane's segment sum to its row of y.  The rows of a
-// sub-step are runs of consecutive lanes, each at most nsr long (a row has
-// nsr segments): a segmented shuffle reduction with as many steps as the
-// longest run needs leaves each row's sum in its first lane.
-__device__ __forceinline__ void row_add(int64_t acc, uint32_t row, uint32_t nsr, int64_t* ys,
-                                        int lane) {
-  const uint32_t span = nsr < 32 ? nsr : 32;
-  long long s = acc;
-  for (uint32_t d = 1; d < span; d <<= 1) {
-    const long long o = __shfl_down_sync(0xffffffffu, s, d);
-    const uint32_t ro = __shfl_down_sync(0xffffffffu, row, d);
-    if (lane + d < 32 && ro == row) s += o;
-  }
-  const uint32_t rprev = __shfl_up_sync(0xffffffffu, row, 1);
-  if (row != 0xffffffffu && (lane == 0 || rprev != row) && s)
-    atomicAdd(reinterpret_cast<unsigned long long*>(ys + row), (unsigned long long)s);
-}
-
-// One stage of a matrix at compile-time width B: segments [g0, g1) whose
-// words start at word w_lo of A, staged at shared address `sp`; n columns,
-// nsr segments per row (divided by dm, ds & 255, ds >> 8).
-template <int B, bool SGN, bool FAST>
-__device__ __noinline__ void run_stage(uint32_t sp, uint64_t w_lo, uint32_t g0, uint32_t g1,
-                                       uint32_t n, uint32_t nsr, uint32_t dm, uint32_t ds,
-                                       const int* ximg, int64_t* ys) {
-  const int lane = threadIdx.x % 32;
-  const uint32_t ds1 = ds & 255u, ds2 = ds >> 8;
-  // Fast path: each lane keeps a running sum for its current row and adds it
-  // to y (one atomic, no warp-wide step) when its next segment starts another
-  // row and at the end of the stage.  General path: rows reduced per sub-step.
-  int64_t racc = 0;
-  uint32_t rrow = 0xffffffffu;
-  for (uint32_t base = g0; base < g1; base += 32) {
-    const uint32_t g = base + lane;
-    const bool live = g < g1;
-    const uint32_t gg = live ? g : base;  // a dead lane decodes a live segment, then drops it
-    const uint32_t q = div_seg(gg, dm, ds1, ds2);
-    const uint32_t s = gg - q * nsr;
-    const uint64_t bit = ((uint64_t)q * n + 32u * s) * (uint64_t)B;
-    const uint32_t wo = (uint32_t)((bit >> 5) - w_lo), sh = (uint32_t)bit & 31u;
-    if constexpr (FAST) {
-      const int4* xb = reinterpret_cast<const int4*>(ximg);
-      const int4 x0 = __ldg(xb + s), x1 = __ldg(xb + nsr + s);
-      const int xs = SGN ? __ldg(ximg + 8 * nsr + s) : 0;
-      uint32_t f[B + 1];
-      load_segment<B>(sp, wo, sh, f);
-      flip_signs<B, SGN>(f);
-      const int xw[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-      const int64_t acc = seg_dot_fast<B, SGN>(f, xw, xs);
-      if (live) {
-        if (q != rrow) {
-          if (racc) atomicAdd(reinterpret_cast<unsigned long long*>(ys + rrow), (unsigned long long)racc);
-          rrow = q;
-          racc = acc;
-        } else {
-          racc += acc;
-        }
-      }
-    } else {
-      uint32_t f[B + 1];
-      load_segment<B>(sp, wo, sh, f);
-      int64_t acc = seg_dot_gen<B, SGN>(f, reinterpret_cast<const int4*>(ximg) + s, nsr);
-      if (!live) acc = 0;
-      row_add(acc, live ? q : 0xffffffffu, nsr, ys, lane);
-    }
-  }
-  if (FAST && racc) atomicAdd(reinterpret_cast<unsigned long long*>(ys + rrow), (unsigned long long)racc);
 }
 
 // Re-pack y of one matrix at its exact width; the whole warp takes part
@@ -400,199 +251,78 @@ __device__ void pack_y_warp(const Mat& M, const int64_t* __restrict__ ys, int la
 // ---------------------------------------------------------------------------
 // The persistent kernel
 // ---------------------------------------------------------------------------
-// A staged stage, written by lane 0 when it issues the copy: everything the
-// decode needs, so that the consumer reads no descriptor from global memory.
-__device__ __forceinline__ uint32_t lo32(const void* p) { return (uint32_t)(uintptr_t)p; }
-__device__ __forceinline__ uint32_t hi32(const void* p) { return (uint32_t)((uintptr_t)p >> 32); }
-template <typename T>
-__device__ __forceinline__ T* ptr_of(uint32_t lo, uint32_t hi) {
-  return reinterpret_cast<T*>(((uint64_t)hi << 32) | lo);
-}
-
-// A staged stage (64 bytes in shared memory, written by lane 0 with four
-// 16-byte stores when it issues the copy, read back the same way): all the
-// decode needs, so that the consumer reads nothing else.
-//   q[0]: w_lo (first word of the slot's copy), x image
-//   q[1]: y scratch rows, g0, g1 (segments)
-//   q[2]: n, nsr, dm, ds (ds1 | ds2 << 8)
-//   q[3]: code, matrix, last stage of its unit, 0
-struct alignas(16) Desc {
-  uint4 q[4];
+// A unit with its matrix, as lane 0 fetches it for its warp.
+struct alignas(16) Job {
+  MatView view;
+  uint32_t seg0, nseg, code, mat;
+  uint32_t units;  // of the matrix; 0: no unit left
 };
-
-// The unit a warp is issuing (64 bytes in shared memory, written by lane 0
-// when the warp takes the unit, read by the producer per stage).
-//   q[0]: A's words, x image     q[1]: y scratch rows, n, nsr
-//   q[2]: dm, ds, code, matrix   q[3]: seg0, nseg, 0, 0
-struct alignas(16) URec {
-  uint4 q[4];
-};
-
-// The stage producer of one warp: every lane holds the same state; lane 0
-// takes the tickets, fills the unit record and issues the copies.
-struct Producer {
-  uint32_t unit;   // unit being issued (>= nunits: none left)
-  uint32_t pos;    // its segments already issued
-  uint32_t nseg;   // its segments
-  uint32_t tk;     // lane 0: the ticket taken one unit ahead
-  uint32_t count;  // units to hand out (the valid entries')
-
-  __device__ __forceinline__ void take(const Args& a, URec* rec, int lane) {
-    const uint32_t t = __shfl_sync(0xffffffffu, tk, 0);
-    pos = 0;
-    unit = a.nunits;
-    if (t < count) {
-      if (lane == 0) {
-        tk = atomicAdd(a.ticket, 1u);  // (its latency hides behind the loads below)
-        const uint32_t ui = a.order[t];
-        const Unit u = a.units[ui];
-        const Mat& M = a.mats[u.mat];
-        const uint32_t code = a.codes[u.mat];
-        const int* ximg = a.ximage + M.x_off;
-        int64_t* ys = a.yscratch + M.y_off;
-        rec->q[0] = make_uint4(lo32(M.wa), hi32(M.wa), lo32(ximg), hi32(ximg));
-        rec->q[1] = make_uint4(lo32(ys), hi32(ys), M.n, M.nseg_row);
-        rec->q[2] = make_uint4(M.dm, M.ds1 | (M.ds2 << 8), code, u.mat);
-        rec->q[3] = make_uint4(u.seg0, u.nseg, ui, 0);
-      }
-      __syncwarp();
-      const uint4 r3 = rec->q[3];
-      unit = r3.z;
-      nseg = r3.y;
-    }
-  }
-
-  // Issues the next stage into slot memory `dst` (false: no stage left).
-  __device__ __forceinline__ bool issue(const Args& a, uint8_t* dst, uint64_t* bar, Desc* d,
-                                        URec* rec, int lane) {
-    if (unit >= a.nunits) return false;
-    const uint4 r0 = rec->q[0], r1 = rec->q[1], r2 = rec->q[2], r3 = rec->q[3];
-    const uint32_t n = r1.z, nsr = r1.w, dm = r2.x, ds = r2.y, code = r2.z;
-    const int b = code_width(code);
-    const uint32_t cnt = umin(nseg - pos, 32u * code_lane_segs(code));
-    const uint32_t g0 = r3.x + pos, g1 = g0 + cnt;
-    uint64_t w_lo = 0;
-    uint32_t bytes = 0;
-    if (cnt) {
-      const uint32_t ds1 = ds & 255u, ds2 = ds >> 8;
-      const uint32_t q0 = div_seg(g0, dm, ds1, ds2), s0 = g0 - q0 * nsr;
-      const uint32_t ql = div_seg(g1 - 1, dm, ds1, ds2), sl = g1 - 1 - ql * nsr;
-      const uint64_t fb = ((uint64_t)q0 * n + 32u * s0) * (uint64_t)b;
-      const uint64_t eb = ((uint64_t)ql * n + umin(n, 32u * sl + 32u)) * (uint64_t)b;
-      w_lo = (fb >> 5) & ~3ull;
-      const uint64_t w_hi = (((eb + 31) >> 5) + 3) & ~3ull;
-      bytes = (uint32_t)((w_hi - w_lo) * 4);
-    }
-    pos += cnt;
-    const bool last = pos >= nseg;
-    if (lane == 0) {
-      d->q[0] = make_uint4((uint32_t)w_lo, (uint32_t)(w_lo >> 32), r0.z, r0.w);
-      d->q[1] = make_uint4(r1.x, r1.y, g0, g1);
-      d->q[2] = make_uint4(n, nsr, dm, ds);
-      d->q[3] = make_uint4(code, r2.w, last ? 1u : 0u, 0u);
-      ax::mbar_expect_tx(bar, bytes);
-      if (bytes) ax::bulk_g2s(dst, ptr_of<const uint32_t>(r0.x, r0.y) + w_lo, bytes, bar);
-    }
-    if (last) take(a, rec, lane);
-    return true;
-  }
-};
-
-__device__ __forceinline__ void stage_dispatch(uint32_t sp, const uint4 (&d)[4]) {
-  const uint64_t w_lo = ((uint64_t)d[0].y << 32) | d[0].x;
-  const int* ximg = ptr_of<const int>(d[0].z, d[0].w);
-  int64_t* ys = ptr_of<int64_t>(d[1].x, d[1].y);
-  const uint32_t g0 = d[1].z, g1 = d[1].w, n = d[2].x, nsr = d[2].y, dm = d[2].z, ds = d[2].w;
-  switch (d[3].x & 0x1ffu) {
-#define CCM_BT_GEN(B)                                                          \
-  case (B): run_stage<B, false, false>(sp, w_lo, g0, g1, n, nsr, dm, ds, ximg, ys); break; \
-  case (B) | 128: run_stage<B, true, false>(sp, w_lo, g0, g1, n, nsr, dm, ds, ximg, ys); break;
-#define CCM_BT_FAST(B)                                                         \
-  case (B) | 256: run_stage<B, false, true>(sp, w_lo, g0, g1, n, nsr, dm, ds, ximg, ys); break; \
-  case (B) | 384: run_stage<B, true, true>(sp, w_lo, g0, g1, n, nsr, dm, ds, ximg, ys); break;
-#define CCM_BT_BOTH(B) CCM_BT_GEN(B) CCM_BT_FAST(B)
-    CCM_BT_BOTH(1) CCM_BT_BOTH(2) CCM_BT_BOTH(3) CCM_BT_BOTH(4) CCM_BT_BOTH(5) CCM_BT_BOTH(6)
-    CCM_BT_BOTH(7) CCM_BT_BOTH(8) CCM_BT_BOTH(9) CCM_BT_BOTH(10) CCM_BT_BOTH(11) CCM_BT_BOTH(12)
-    CCM_BT_BOTH(13) CCM_BT_BOTH(14) CCM_BT_BOTH(15) CCM_BT_BOTH(16) CCM_BT_BOTH(17) CCM_BT_BOTH(18)
-    CCM_BT_BOTH(19) CCM_BT_BOTH(20) CCM_BT_BOTH(21) CCM_BT_BOTH(22) CCM_BT_BOTH(23) CCM_BT_BOTH(24)
-    CCM_BT_GEN(25) CCM_BT_GEN(26) CCM_BT_GEN(27) CCM_BT_GEN(28) CCM_BT_GEN(29) CCM_BT_GEN(30)
-    CCM_BT_GEN(31) CCM_BT_GEN(32)
-#undef CCM_BT_BOTH
-#undef CCM_BT_FAST
-#undef CCM_BT_GEN
-    default: break;
-  }
-}
 
 // Dynamic shared memory: each warp's D ring slots.
 __global__ void __launch_bounds__(kThreads, 3) k_batch_mv(const __grid_constant__ Args a) {
   extern __shared__ __align__(128) uint8_t s_ring[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][kMaxSlots];
-  __shared__ Desc s_desc[kWarps][kMaxSlots];
-  __shared__ URec s_rec[kWarps];
+  __shared__ Job s_job[kWarps];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const uint32_t D = a.slots, SB = a.slot_bytes;
-  uint8_t* ring = s_ring + (size_t)warp * D * SB;
-  uint64_t* bar = s_bar[warp];
-  Desc* desc = s_desc[warp];
-  URec* rec = &s_rec[warp];
-  if (lane == 0) {
-    for (uint32_t s = 0; s < D; ++s) ax::mbar_init(&bar[s], 1);
-    ax::mbar_init_fence();
-  }
+  Ring ring{s_ring + (size_t)warp * a.slots * a.slot_bytes, s_bar[warp], a.slot_bytes, a.slots,
+            a.stage_bytes, 0, 0};
+  ring.init(lane);
+  const uint32_t count = a.order[a.nunits];  // units to hand out (the valid entries')
+  uint32_t ticket = 0;                       // lane 0: the next unit's
+  if (lane == 0) ticket = atomicAdd(a.ticket, 1u);
+  // Lane 0: the unit of `ticket` into the warp's job.
+  auto fetch = [&] {
+    if (lane == 0) {
+      Job j{};
+      if (ticket < count) {
+        const Unit u = a.units[a.order[ticket]];
+        const Mat& M = a.mats[u.mat];
+        j.view = MatView{M.wa, reinterpret_cast<const uint8_t*>(a.ximage + M.x_off),
+                         a.yscratch + M.y_off, M.n, M.nseg_row, M.dm, M.ds1, M.ds2};
+        j.seg0 = u.seg0;
+        j.nseg = u.nseg;
+        j.code = a.codes[u.mat];
+        j.mat = u.mat;
+        j.units = M.units;
+      }
+      s_job[warp] = j;
+    }
+  };
+  fetch();
   __syncwarp();
-  Producer pr;
-  pr.count = a.order[a.nunits];
-  if (lane == 0) pr.tk = atomicAdd(a.ticket, 1u);
-  pr.take(a, rec, lane);
-  uint32_t issued = 0;
-  while (issued < D && pr.issue(a, ring + issued * SB, &bar[issued], &desc[issued], rec, lane))
-    ++issued;
-  uint32_t consumed = 0, slot = 0, phase = 0;
-  bool ok = true;
-  while (consumed < issued) {
-    if (!ax::mbar_wait(&bar[slot], phase)) {
-      ok = false;
+  Job job = s_job[warp];
+  while (job.units) {
+    auto next = [&] {
+      if (lane == 0) ticket = atomicAdd(a.ticket, 1u);
+      fetch();
+    };
+    bool ok = true;
+    if (job.nseg)
+      ok = matrix_range(job.view, ring, job.seg0, job.seg0 + job.nseg, code_width(job.code),
+                        code_signed(job.code), code_mode(job.code), next);
+    else
+      next();
+    if (!ok) {
+      // a wait gave up: mark the entries whose units this warp holds
+      if (lane == 0) {
+        set_status(a.mats[job.mat].hy, CCM_E_TIMEOUT);
+        if (s_job[warp].units) set_status(a.mats[s_job[warp].mat].hy, CCM_E_TIMEOUT);
+      }
       break;
     }
-    const uint4 d1 = desc[slot].q[1], d3 = desc[slot].q[3];  // (kept past the decode)
-    if (d1.w > d1.z) {
-      const uint4 d[4] = {desc[slot].q[0], d1, desc[slot].q[2], d3};
-      stage_dispatch(ax::smem_u32(ring + slot * SB), d);
+    // the unit is complete; the warp completing a matrix packs its y
+    __threadfence();
+    __syncwarp();
+    uint32_t fin = 0;
+    if (lane == 0) fin = atomicAdd(a.done + job.mat, 1u) + 1 == job.units;
+    fin = __shfl_sync(0xffffffffu, fin, 0);
+    if (fin) {
+      __threadfence();
+      pack_y_warp(a.mats[job.mat], job.view.y, lane);
     }
     __syncwarp();
-    ++consumed;
-    ax::fence_proxy_async_smem();  // this slot's reads before its refill
-    if (pr.issue(a, ring + slot * SB, &bar[slot], &desc[slot], rec, lane)) ++issued;
-    if (d3.z) {
-      // the unit is complete; the warp completing a matrix packs its y
-      const uint32_t dmat = d3.y;
-      __threadfence();
-      __syncwarp();
-      const Mat& M = a.mats[dmat];
-      uint32_t fin = 0;
-      if (lane == 0) fin = atomicAdd(a.done + dmat, 1u) + 1 == M.units;
-      fin = __shfl_sync(0xffffffffu, fin, 0);
-      if (fin) {
-        __threadfence();
-        pack_y_warp(M, ptr_of<int64_t>(d1.x, d1.y), lane);
-      }
-    }
-    if (++slot == D) slot = 0, phase ^= 1;
-  }
-  if (!ok) {
-    // a wait gave up: mark the entries this warp holds units of, and let the
-    // copies still in flight land before the CTA's shared memory goes away
-    for (uint32_t j = consumed; j < issued; ++j) {
-      if (lane == 0) set_status(a.mats[desc[slot].q[3].y].hy, CCM_E_TIMEOUT);
-      if (!ax::mbar_wait(&bar[slot], phase)) {
-        // (a copy that never lands: report and leave it)
-      }
-      if (++slot == D) slot = 0, phase ^= 1;
-    }
-    if (lane == 0 && pr.unit < a.nunits) set_status(a.mats[rec->q[2].w].hy, CCM_E_TIMEOUT);
-    const uint32_t t = __shfl_sync(0xffffffffu, pr.tk, 0);
-    if (lane == 0 && t < pr.count) set_status(a.mats[a.units[a.order[t]].mat].hy, CCM_E_TIMEOUT);
+    job = s_job[warp];
+    __syncwarp();
   }
 }
 
@@ -790,7 +520,7 @@ ccm_status ccm_batch_matvec(const void* plan, const ccm_batch_info* info, void* 
   if (info->stage_bytes != 0 && (info->stage_bytes < 128 || info->stage_bytes > 16384))
     return CCM_E_INVAL;
   a.stage_bytes = info->stage_bytes ? info->stage_bytes : kDefaultStageBytes;
-  a.slot_bytes = slot_bytes(a.stage_bytes, (int)a.bmax);
+  a.slot_bytes = ccm::seg::slot_bytes(a.stage_bytes, (int)a.bmax);
   // warps per CTA: 8, or 4 when that keeps more warps resident per SM (the
   // rings are per warp, so a smaller CTA packs the shared memory tighter)
   static size_t attr = 0;
@@ -824,8 +554,11 @@ ccm_status ccm_batch_matvec(const void* plan, const ccm_batch_info* info, void* 
   const size_t smem = (size_t)warps * a.slots * a.slot_bytes;
   if (grid <= 0) grid = ccm::num_sms() * per;  // one resident wave
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  k_batch_init<<<info->count, 256, 0, st>>>(a);
-  k_batch_order<<<1, kOrderThreads, 0, st>>>(a);
+  k_batch_init<<<info->count, kInitThreads, 0, st>>>(a);
+  // (a slice of at least 64 entries per CTA)
+  const unsigned order_grid =
+      (unsigned)ccm::umax(1, ccm::umin((info->count + 63) / 64, (uint64_t)ccm::num_sms()));
+  k_batch_order<<<order_grid, kOrderThreads, 0, st>>>(a);
   ccm::profile_begin(st);
   k_batch_mv<<<grid, 32 * warps, smem, st>>>(a);
   ccm::profile_end(st);
