@@ -1,5 +1,5 @@
 // ew_kernels.cuh -- elementwise kernels on the group engine: SM pack of dense
-// int32/int64 data, unpack, and the add / scale operations whose results are
+// int32/int64 data and the add / scale operations whose results are
 // re-packed at their own width.  Each is instantiated per width class
 // (ew8.cu, ew16.cu, ew32.cu); the host picks the class from the widths the
 // buffer capacities allow.
@@ -1190,60 +1190,24 @@ inline size_t pack_ws_bytes(uint64_t n, int cls) {
   return ((ntiles * 32 * cls * 4 + 255) & ~(size_t)255) + ((ntiles + 255) & ~(size_t)255);
 }
 
-// Unpack: decode every group and write the values densely (int64 or int32).
-template <typename T, int BMAX>
-__global__ void __launch_bounds__(kThreads) k_unpack_ge(const ccm_header* h,
-                                                        const uint32_t* __restrict__ w,
-                                                        uint64_t rows, uint64_t cols,
-                                                        uint64_t capacity, T* __restrict__ out,
-                                                        int32_t* err) {
-  __shared__ __align__(16) uint32_t s_buf[kWarps][kBufWords];
-  int st = check_input(h, rows, cols, capacity);
-  const int b = h->width, sgn = h->is_signed;
-  if (st == CCM_OK && sizeof(T) == 4 && (sgn ? b > 32 : b > 31)) st = CCM_E_WIDTH;
-  if (err && blockIdx.x == 0 && threadIdx.x == 0) *err = st;
-  if (st != CCM_OK) return;
-  const uint64_t n = rows * cols;
-  const uint64_t dw = data_words(n, b);
-  const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
-  uint32_t* buf = s_buf[warp];
-  T* tb = reinterpret_cast<T*>(buf);
-  const uint64_t ntiles = (n + kTile - 1) / kTile;
-  const uint64_t gwarps = (uint64_t)gridDim.x * kWarps;
-  for (uint64_t tile = (uint64_t)blockIdx.x * kWarps + warp; tile < ntiles; tile += gwarps) {
-    const uint32_t nt = (uint32_t)umin((uint64_t)kTile, n - tile * kTile);
-    stage_packed(buf, w, tile, b, dw, lane);
-    __syncwarp();
-    int64_t v[32];
-    decode_dispatch<BMAX>(b, sgn, buf, lane, [&](int k, int64_t x) { v[k] = x; });
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < 32; ++k) tb[33 * lane + k] = (T)v[k];
-    __syncwarp();
-    store_dense<T>(tb, out, tile * kTile, nt, lane);
-    __syncwarp();
-  }
-}
-
 // What the host asks one class to run.
 enum class EwKind {
-  PackI64, PackI32, AddStats, AddSpec, AddPack, ScaleStats, ScaleSpec, ScalePack, UnpackI64,
-  UnpackI32, LocalI64, LocalI32, Repack
+  PackI64, PackI32, AddStats, AddSpec, AddPack, ScaleStats, ScaleSpec, ScalePack, LocalI64,
+  LocalI32, Repack
 };
 
 struct EwCall {
   EwKind kind;
-  const void* dense;      // PackI64 / PackI32 source, Unpack destination
+  const void* dense;      // PackI64 / PackI32 source
   const ccm_header* ha;   // packed inputs
   const uint32_t* wa;
   const ccm_header* hb;
   const uint32_t* wb;
   int64_t s;              // scale factor
-  ccm_header* out;        // output header (pack/stats) or input header (unpack)
-  uint32_t* words;        // output words, or input words (unpack)
+  ccm_header* out;        // output header
+  uint32_t* words;        // output words
   uint64_t capacity;
   uint64_t rows, cols;
-  int32_t* err;           // unpack status
   void* ws;               // Local* / Repack: workspace (slots, then tile widths)
   int slot_class;         // Local* / Repack: width class of the output (slot = 32*class words)
   int spec;               // AddPack / ScalePack: an AddSpec / ScaleSpec launch came first;
@@ -1311,7 +1275,7 @@ int launch_ew_scale(const EwCall& c, cudaStream_t st) {
   return launched;
 }
 
-// PackI64 / PackI32 / LocalI64 / LocalI32 / Repack / UnpackI64 / UnpackI32
+// PackI64 / PackI32 / LocalI64 / LocalI32 / Repack
 template <int C>
 int launch_ew_pack(const EwCall& c, cudaStream_t st) {
   const uint64_t n = c.rows * c.cols;
@@ -1368,14 +1332,6 @@ int launch_ew_pack(const EwCall& c, cudaStream_t st) {
       }
       break;
     }
-    case EwKind::UnpackI64:
-      k_unpack_ge<int64_t, C><<<ew_grid(n, 12), kThreads, 0, st>>>(
-          c.out, c.words, c.rows, c.cols, c.capacity, (int64_t*)c.dense, c.err);
-      break;
-    case EwKind::UnpackI32:
-      k_unpack_ge<int32_t, C><<<ew_grid(n, 12), kThreads, 0, st>>>(
-          c.out, c.words, c.rows, c.cols, c.capacity, (int32_t*)c.dense, c.err);
-      break;
     default:
       return 0;
   }

@@ -89,16 +89,6 @@ __device__ __forceinline__ void stage_dense(T* buf, const T* __restrict__ src, u
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void store_dense(const T* buf, T* __restrict__ dst, uint64_t base,
-                                            uint32_t nt, int lane) {
-#pragma unroll 8
-  for (int j = 0; j < 32; ++j) {
-    uint32_t f = lane + 32 * j;
-    if (f < nt) dst[base + f] = buf[f + (f >> 5)];
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Compile-time width: decode the lane's group (32 fields of width B) and hand
 // each value to fn(k, value) with k a compile-time index.

@@ -300,32 +300,106 @@ __global__ void __launch_bounds__(256) k_unpack(const ccm_header* h, const uint3
     out[i] = (T)decode_field(w, i, b, sgn);
 }
 
-void run_unpack(const ccm_matrix& a, void* dense, int dtype, int32_t* err, cudaStream_t st) {
-  uint64_t n = a.rows * a.cols;
-  const int cls = ew_class(width_bound(a.capacity, n));
-  if (cls && n) {
-    ge::EwCall c{};
-    c.kind = dtype == CCM_I64 ? ge::EwKind::UnpackI64 : ge::EwKind::UnpackI32;
-    c.dense = dense;
-    c.out = a.hdr;
-    c.words = a.words;
-    c.capacity = a.capacity;
-    c.rows = a.rows;
-    c.cols = a.cols;
-    c.err = err;
-    profile_begin(st);
-    launch_ew(cls, c, st);
-    profile_end(st);
-    return;
+// Fields of at most 32 bits to a dense matrix.  A warp unpacks runs of 512 fields (16 b whole words): lane l takes
+// the pairs 2 l + 64 j, so a lane's shift is fixed and its words lie 2 b apart,
+// every load is one of 24 issued together, and each warp store writes 64
+// consecutive entries (as pairs where the destination is aligned to them).  A
+// full run may read up to two words of the next one, which exist (the words
+// are padded to four).  Bound by HBM (b/8 bytes in, the entry out).  Measured
+// on GB300 (8192^2 at 12 bits to int64; before: a group of 32 fields per lane
+// through shared memory, 8 warps per SM): 122 -> 103 us (6.2 TB/s).
+constexpr int kUnpackPairs = 8;                      // per lane and run
+constexpr int kUnpackRun = 64 * kUnpackPairs;        // fields
+
+template <typename T>
+struct Pair;
+template <>
+struct Pair<int64_t> { using type = longlong2; };
+template <>
+struct Pair<int32_t> { using type = int2; };
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_unpack_pairs(const ccm_header* h,
+                                                      const uint32_t* __restrict__ w, uint64_t rows,
+                                                      uint64_t cols, uint64_t capacity,
+                                                      T* __restrict__ out, int32_t* err) {
+  const HeaderView hv = load_header(h);
+  int st = check_header(hv, rows, cols, capacity);
+  const int b = hv.width, sgn = hv.is_signed;
+  if (st == CCM_OK && sizeof(T) == 4 && (sgn ? b > 32 : b > 31)) st = CCM_E_WIDTH;
+  if (st == CCM_OK && b > 32) st = CCM_E_INPUT;  // (the capacity bounds b by 32)
+  if (err && blockIdx.x == 0 && threadIdx.x == 0) *err = st;
+  if (st != CCM_OK) return;
+  using V = typename Pair<T>::type;
+  const uint64_t n = rows * cols, dw = data_words(n, b);
+  const int lane = threadIdx.x % 32, sh = 32 - b;
+  const uint32_t bit = 2 * lane * b, at = bit & 31;
+  const uint64_t runs = (n + kUnpackRun - 1) / kUnpackRun, warps = (uint64_t)gridDim.x * 8;
+  const bool pairs = reinterpret_cast<uintptr_t>(out) % sizeof(V) == 0;
+  auto low = [&](uint32_t x) {  // the low b bits as an entry
+    const uint32_t t = x << sh;
+    return sgn ? (T)((int)t >> sh) : (T)(t >> sh);
+  };
+  for (uint64_t r = (uint64_t)blockIdx.x * 8 + threadIdx.x / 32; r < runs; r += warps) {
+    const uint64_t w0 = r * (uint64_t)(16 * b) + (bit >> 5);
+    const uint64_t e0 = r * kUnpackRun + 2 * lane;
+    if (r + 1 < runs) {
+      const uint32_t* p = w + w0;
+      uint32_t x[kUnpackPairs][3];
+#pragma unroll
+      for (int j = 0; j < kUnpackPairs; ++j, p += 2 * b)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) x[j][q] = __ldg(p + q);
+#pragma unroll
+      for (int j = 0; j < kUnpackPairs; ++j) {
+        const uint32_t lo = __funnelshift_r(x[j][0], x[j][1], at);
+        const uint32_t hi = __funnelshift_r(x[j][1], x[j][2], at);
+        V v;
+        v.x = low(lo);
+        v.y = low(__funnelshift_rc(lo, hi, b));
+        if (pairs) {
+          __stcs(reinterpret_cast<V*>(out + e0) + 32 * j, v);
+        } else {
+          out[e0 + 64 * j] = v.x;
+          out[e0 + 64 * j + 1] = v.y;
+        }
+      }
+    } else {
+      // the last run: no word past the data, no entry past the end
+      for (int j = 0; j < kUnpackPairs; ++j) {
+        const uint64_t wj = w0 + (uint64_t)(2 * b) * j, e = e0 + 64 * j;
+        uint32_t x[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) x[q] = wj + q < dw ? __ldg(w + wj + q) : 0u;
+        const uint32_t lo = __funnelshift_r(x[0], x[1], at), hi = __funnelshift_r(x[1], x[2], at);
+        if (e < n) out[e] = low(lo);
+        if (e + 1 < n) out[e + 1] = low(__funnelshift_rc(lo, hi, b));
+      }
+    }
   }
-  int grid = (int)umin(umax((n + 255) / 256, 1), (uint64_t)num_sms() * 16);
+}
+
+void run_unpack(const ccm_matrix& a, void* dense, int dtype, int32_t* err, cudaStream_t st) {
+  const uint64_t n = a.rows * a.cols;
   profile_begin(st);
-  if (dtype == CCM_I64)
-    k_unpack<int64_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
-                                            (int64_t*)dense, err);
-  else
-    k_unpack<int32_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
-                                            (int32_t*)dense, err);
+  if (n && width_bound(a.capacity, n) <= 32) {
+    const uint64_t runs = (n + kUnpackRun - 1) / kUnpackRun;
+    const int grid = (int)umin((runs + 7) / 8, (uint64_t)num_sms() * 16);
+    if (dtype == CCM_I64)
+      k_unpack_pairs<int64_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
+                                                    (int64_t*)dense, err);
+    else
+      k_unpack_pairs<int32_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
+                                                    (int32_t*)dense, err);
+  } else {
+    const int grid = (int)umin(umax((n + 255) / 256, 1), (uint64_t)num_sms() * 16);
+    if (dtype == CCM_I64)
+      k_unpack<int64_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
+                                              (int64_t*)dense, err);
+    else
+      k_unpack<int32_t><<<grid, 256, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity,
+                                              (int32_t*)dense, err);
+  }
   profile_end(st);
   note_launch();
 }
