@@ -9,6 +9,7 @@
 // entries before it.  On the GPU the encoder is therefore a scan --
 //   k_vlb_lens   per 1024-entry block: sum of L, global max of L
 //   k_vlb_scan   one CTA: k, block bit offsets (exclusive scan), header
+//   k_vlb_zero   the words that two blocks share
 //   k_vlb_write  per block: in-block scan of k + L, bits assembled in shared
 //                memory, interior words stored, the two boundary words OR-ed
 // -- and it also writes an index: the bit offset of every 64th entry (plus
@@ -131,12 +132,19 @@ __global__ void __launch_bounds__(1024) k_vlb_scan(uint64_t* __restrict__ block_
   }
 }
 
-__global__ void k_vlb_zero(const ccm_header* hdr, uint32_t* __restrict__ words, uint64_t capacity) {
+// Zeroes the words that more than one block ORs its bits into (the first one of
+// every block) and the padding; k_vlb_write stores every other word whole.
+// (Clearing the whole stream first: 9 us for 52 MB, now 2.)
+__global__ void __launch_bounds__(256) k_vlb_zero(const ccm_header* hdr,
+                                                  uint32_t* __restrict__ words,
+                                                  const uint64_t* __restrict__ block_off,
+                                                  uint64_t nblocks) {
   if (hdr->status != CCM_OK) return;
-  const uint64_t nw = umin(hdr->nwords, capacity);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    words[i] = 0;
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < nblocks;
+       i += (uint64_t)gridDim.x * 256)
+    words[block_off[i] / 32] = 0;
+  if (blockIdx.x == 0)  // the last block's last word, and the padding after it
+    for (uint64_t w = hdr->stat_or / 32 + threadIdx.x; w < hdr->nwords; w += 256) words[w] = 0;
 }
 
 template <typename T>
@@ -209,7 +217,7 @@ __global__ void __launch_bounds__(kThreads) k_vlb_write(const T* __restrict__ sr
     const uint32_t nwords_blk = (uint32_t)((shift0 + block_bits + 31) / 32);
     for (uint32_t i = threadIdx.x; i < nwords_blk; i += kThreads) {
       const uint32_t val = s_words[i];
-      if (i == 0 || i == nwords_blk - 1)
+      if (i == 0 || (i == nwords_blk - 1 && (shift0 + block_bits) % 32))
         atomicOr(&words[w0 + i], val);  // shared with the neighbouring blocks
       else
         words[w0 + i] = val;
@@ -905,8 +913,8 @@ void run_vlb_pack(const void* dense, int dtype, uint64_t rows, uint64_t cols, cc
                                       index, entries);
   note_launch(2);
   if (!words) return;
-  vlb::k_vlb_zero<<<(int)umin((capacity + 255) / 256 + 1, (uint64_t)num_sms() * 8), 256, 0, st>>>(
-      hdr, words, capacity);
+  vlb::k_vlb_zero<<<(int)umin(nblocks / 256 + 1, (uint64_t)num_sms() * 4), 256, 0, st>>>(
+      hdr, words, block, nblocks);
   profile_begin(st);
   if (dtype == CCM_I64)
     vlb::k_vlb_write<int64_t><<<g, vlb::kThreads, 0, st>>>((const int64_t*)dense, n, block, hdr,
