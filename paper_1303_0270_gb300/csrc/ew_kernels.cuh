@@ -924,6 +924,14 @@ __device__ __forceinline__ void st_relaxed_gpu(uint64_t* p, uint64_t v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(v));
 }
 
+// Merges width statistics into the header, without an atomic where the header
+// holds them already.
+__device__ __forceinline__ void merge_stats(ccm_header* out, uint64_t orv, uint32_t neg) {
+  if (orv & ~ld_relaxed_gpu(&out->stat_or))
+    atomicOr(reinterpret_cast<unsigned long long*>(&out->stat_or), (unsigned long long)orv);
+  if (neg && !*reinterpret_cast<volatile uint32_t*>(&out->stat_neg)) atomicOr(&out->stat_neg, 1u);
+}
+
 __device__ __forceinline__ void issue_dense_tile(int64_t* dst, const int64_t* __restrict__ src,
                                                  uint64_t base, uint32_t nt, int lane) {
 #pragma unroll 4
@@ -992,12 +1000,21 @@ __global__ void __launch_bounds__(kThreads) k_pack_local(const T* __restrict__ s
   uint32_t g_neg = 0;
   int cur = 0;
   // the speculation flag as this warp last saw it (sticky once set, so a
-  // warp stops reading it after the first time it finds it set)
-  bool known = exact;
+  // warp stops reading it after the first time it finds it set).  Stores to one
+  // word are served one after the other (7,296 warps, each storing the flag for
+  // its first tile: 50 us), so one CTA in 16 stores it at once and the others
+  // only if they still find it clear at their next tile; it only saves slots
+  bool known = exact, pending = false;
+  const bool herald = blockIdx.x % 16 == 0 && warp == 0;
   for (; tile < ntiles; tile += gwarps) {
     const uint32_t nt = (uint32_t)umin((uint64_t)kTile, n - tile * kTile);
     // (read before the tile's wait so that its latency hides behind it)
-    if (b_spec && !known) known = ld_relaxed_gpu(&out->reserved1) != 0;
+    if (b_spec && !known)
+      known = ld_relaxed_gpu(&out->reserved1) != 0;
+    else if (pending) {
+      if (lane == 0 && ld_relaxed_gpu(&out->reserved1) == 0) st_relaxed_gpu(&out->reserved1, 1ull);
+      pending = false;
+    }
     int64_t v[32];
     {
       const uint64_t next = tile + gwarps;
@@ -1046,7 +1063,10 @@ __global__ void __launch_bounds__(kThreads) k_pack_local(const T* __restrict__ s
     // the slot is needed unless the matrix width is known to be b_spec
     bool slot = true;
     if (b_spec) {
-      if (!exact && bl == b_spec && !known && lane == 0) st_relaxed_gpu(&out->reserved1, 1ull);
+      if (!exact && bl == b_spec && !known) {
+        if (herald && lane == 0) st_relaxed_gpu(&out->reserved1, 1ull);
+        pending = !herald;
+      }
       slot = !(known || bl == b_spec);
       known = known || bl == b_spec;
     }
@@ -1082,9 +1102,21 @@ __global__ void __launch_bounds__(kThreads) k_pack_local(const T* __restrict__ s
     if (lane == 0 && tile_width) tile_width[tile] = fits ? (uint8_t)(bl | (neg ? 0x80 : 0)) : 0xFF;
   }
   cp_async_wait0_ge();
+  if (exact) return;  // (the statistics are complete)
+  // one merge per CTA, of the bits that the header does not hold yet
+  __shared__ uint64_t s_or[kWarps];
+  __shared__ uint32_t s_neg[kWarps];
   if (lane == 0) {
-    if (g_or) atomicOr(reinterpret_cast<unsigned long long*>(&out->stat_or), (unsigned long long)g_or);
-    if (g_neg) atomicOr(&out->stat_neg, 1u);
+    s_or[warp] = g_or;
+    s_neg[warp] = g_neg;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kWarps; ++w) {
+      g_or |= s_or[w];
+      g_neg |= s_neg[w];
+    }
+    merge_stats(out, g_or, g_neg);
   }
 }
 
