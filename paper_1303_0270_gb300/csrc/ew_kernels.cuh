@@ -547,6 +547,25 @@ struct OpScale {
 // and returns after the header when the exact width is the speculative one.
 constexpr int kStats = 0, kPack = 1, kSpec = 2;
 
+// Relaxed loads and stores at GPU scope (the speculation flag: written by
+// some warps, read by all; no ordering needed beyond eventual visibility).
+__device__ __forceinline__ uint64_t ld_relaxed_gpu(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_gpu(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(v));
+}
+
+// Merges width statistics into the header, without an atomic where the header
+// holds them already.
+__device__ __forceinline__ void merge_stats(ccm_header* out, uint64_t orv, uint32_t neg) {
+  if (orv & ~ld_relaxed_gpu(&out->stat_or))
+    atomicOr(reinterpret_cast<unsigned long long*>(&out->stat_or), (unsigned long long)orv);
+  if (neg && !*reinterpret_cast<volatile uint32_t*>(&out->stat_neg)) atomicOr(&out->stat_neg, 1u);
+}
+
 // The speculative pass on lanes, a kernel of its own (few registers, buffers
 // sized to the operands: many warps per SM) launched before k_ew<..., kSpec>:
 // when the operands qualify (Op::lanes_width, decided from the headers), it
@@ -615,6 +634,25 @@ __device__ __noinline__ void lanes_body(const Op& op, ccm_header* out, uint32_t*
     const uint64_t t = tile0 + k * gwarps;
     if (t < ntiles) op.template lanes_fill<B>(t, slot_a(k), slot_a(k) + TW, &bar[k], lane);
   }
+  // Statistics to the header.  Every warp merges into one word, whose atomics
+  // are served one after the other (all at the end, they were the kernel's
+  // tail): one CTA in 16 merges after its first tile, whose bits are nearly
+  // always all there is, and at the end a warp adds only what is not there.
+  const bool herald = blockIdx.x % 16 == 0;
+  auto merge = [&] {
+    uint64_t o;
+    if constexpr (L == 64) {
+      o = warp_or64(orb);
+    } else {
+      constexpr uint32_t slot = BS >= 32 ? ~0u : (1u << BS) - 1u;
+      uint32_t o32 = 0;
+#pragma unroll
+      for (int j = 0; j < KS; ++j) o32 |= (orb32 >> (j * BS)) & slot;
+      o = __reduce_or_sync(0xffffffffu, o32);
+    }
+    const uint32_t ng = __reduce_or_sync(0xffffffffu, neg);
+    if (lane == 0) merge_stats(out, o, ng);
+  };
   uint32_t k = 0;
   bool ok = true;
   for (;; ++k) {
@@ -689,6 +727,7 @@ __device__ __noinline__ void lanes_body(const Op& op, ccm_header* out, uint32_t*
       for (int w = lane; w < tw; w += 32) words[w0 + w] = obuf[w];
     }
     __syncwarp();
+    if (k == 0 && herald) merge();
   }
   if (!ok) {  // a copy that never landed: report it, and wait (bounded) for the rest
     if (lane == 0) set_status(out, CCM_E_TIMEOUT);
@@ -696,21 +735,7 @@ __device__ __noinline__ void lanes_body(const Op& op, ccm_header* out, uint32_t*
       if (tile0 + (k + j) * gwarps < ntiles) ax::mbar_wait(&bar[(k + j) % S], ((k + j) / S) & 1);
     return;
   }
-  uint64_t o;
-  if constexpr (L == 64) {
-    o = warp_or64(orb);
-  } else {
-    constexpr uint32_t slot = BS >= 32 ? ~0u : (1u << BS) - 1u;
-    uint32_t o32 = 0;
-#pragma unroll
-    for (int j = 0; j < KS; ++j) o32 |= (orb32 >> (j * BS)) & slot;
-    o = __reduce_or_sync(0xffffffffu, o32);
-  }
-  const uint32_t ng = __reduce_or_sync(0xffffffffu, neg);
-  if (lane == 0) {
-    if (o) atomicOr(reinterpret_cast<unsigned long long*>(&out->stat_or), (unsigned long long)o);
-    if (ng) atomicOr(&out->stat_neg, 1u);
-  }
+  if (k > 1 || (k == 1 && !herald)) merge();
 }
 
 // Calls lanes_body for the run-time (b, bs, mode).  Add: B <= 32 with
@@ -759,6 +784,8 @@ __global__ void __launch_bounds__(kThreads) k_ew_lanes(Op op, ccm_header* out, u
                                                        uint32_t warp_words) {
   extern __shared__ __align__(16) uint32_t s_lanes[];
   __shared__ uint64_t s_lane_bar[kWarps][3];
+  ax::grid_dep_launch();  // the passes that follow may become resident (they wait)
+  ax::grid_dep_wait();    // the header is initialised
   if (out->status != CCM_OK) return;
   op.init(n);
   const int bs = op.spec_width();
@@ -792,6 +819,7 @@ __global__ void __launch_bounds__(kThreads) k_ew(Op op, ccm_header* out, uint32_
   // after a lane pass or a speculative pass this kernel is launched with
   // programmatic dependent launch: wait for that kernel before reading the
   // header it wrote (a no-op for a normal launch)
+  ax::grid_dep_launch();
   ax::grid_dep_wait();
   int b = 0, sgn = 0;
   if constexpr (MODE == kPack) {
@@ -912,25 +940,6 @@ __global__ void __launch_bounds__(kThreads) k_pack_dense(const T* __restrict__ s
 // Shared layout: element f at f + 2*(f/32) (keeps 16-byte alignment; the
 // lane's 16-byte reads of its 32 elements are conflict-free).
 constexpr int kDensePad = kTile + 2 * (kTile / 32);  // int64 slots per staged tile
-
-// Relaxed loads and stores at GPU scope (the speculation flag: written by
-// some warps, read by all; no ordering needed beyond eventual visibility).
-__device__ __forceinline__ uint64_t ld_relaxed_gpu(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ void st_relaxed_gpu(uint64_t* p, uint64_t v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(v));
-}
-
-// Merges width statistics into the header, without an atomic where the header
-// holds them already.
-__device__ __forceinline__ void merge_stats(ccm_header* out, uint64_t orv, uint32_t neg) {
-  if (orv & ~ld_relaxed_gpu(&out->stat_or))
-    atomicOr(reinterpret_cast<unsigned long long*>(&out->stat_or), (unsigned long long)orv);
-  if (neg && !*reinterpret_cast<volatile uint32_t*>(&out->stat_neg)) atomicOr(&out->stat_neg, 1u);
-}
 
 __device__ __forceinline__ void issue_dense_tile(int64_t* dst, const int64_t* __restrict__ src,
                                                  uint64_t base, uint32_t nt, int lane) {
@@ -1253,6 +1262,17 @@ inline int ew_grid(uint64_t n, int per_sm) {
   return (int)umin(umax(want, 1), (uint64_t)num_sms() * per_sm);
 }
 
+// The grid of a persistent kernel: no more CTAs than stay resident (`per_sm` is
+// kept between calls: the occupancy query is slow next to a launch).
+template <class K>
+int resident_grid(K kernel, size_t smem, int& per_sm, uint64_t n) {
+  if (!per_sm &&
+      (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem) != cudaSuccess ||
+       per_sm < 1))
+    per_sm = 1;
+  return ew_grid(n, per_sm);
+}
+
 // Launchers of one width class C, one per family of EwKind (each family is
 // instantiated in a translation unit of its own so that they compile in
 // parallel).  Each returns the number of kernels launched.  Grids are
@@ -1264,7 +1284,8 @@ int launch_ew_add(const EwCall& c, cudaStream_t st) {
   int launched = 1;
   const uint64_t n = c.rows * c.cols;
   PackedIn a{c.ha, c.wa, 0, 0, 0}, b{c.hb, c.wb, 0, 0, 0};
-  const int g = ew_grid(n, 8);
+  static int per_sm = 0;
+  const int g = resident_grid(k_ew<OpAdd, C, kSpec>, 0, per_sm, n);
   const OpAdd op{a, b};
   if (c.kind == EwKind::AddStats)
     k_ew<OpAdd, C, kStats><<<g, kThreads, 0, st>>>(op, c.out, nullptr, 0, n, 0);
@@ -1288,7 +1309,8 @@ int launch_ew_scale(const EwCall& c, cudaStream_t st) {
   int launched = 1;
   const uint64_t n = c.rows * c.cols;
   const OpScale<SMALL> op{PackedIn{c.ha, c.wa, 0, 0, 0}, c.s};
-  const int g = ew_grid(n, 8);
+  static int per_sm = 0;
+  const int g = resident_grid(k_ew<OpScale<SMALL>, C, kSpec>, 0, per_sm, n);
   if (c.kind == EwKind::ScaleStats) {
     k_ew<OpScale<SMALL>, C, kStats><<<g, kThreads, 0, st>>>(op, c.out, nullptr, 0, n, 0);
   } else if (c.kind == EwKind::ScaleSpec) {

@@ -26,12 +26,16 @@ static void launch_lanes(const Op& op, ccm_header* out, uint32_t* words, uint64_
                          optin - (int)fa.sharedSizeBytes);
     dev_done = dev;
   }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ew_lanes<Op>, kThreads, smem) !=
-          cudaSuccess ||
-      per_sm < 1)
+  // (kept per width bound: the occupancy query is slow next to a launch)
+  static int per_sm_of[33] = {};
+  int& per_sm = per_sm_of[bmax < 0 || bmax > 32 ? 32 : bmax];
+  if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ew_lanes<Op>, kThreads,
+                                                                smem) != cudaSuccess ||
+                  per_sm < 1))
     per_sm = 1;
-  k_ew_lanes<Op><<<ew_grid(n, per_sm), kThreads, smem, st>>>(op, out, words, capacity, n, ww);
+  const int g = ew_grid(n, per_sm);
+  ax::launch_pdl(k_ew_lanes<Op>, dim3(g), dim3(kThreads), smem, st, op, out, words, capacity, n,
+                 ww);
 }
 
 }  // namespace ge
