@@ -165,8 +165,9 @@ size_t pack_workspace(uint64_t rows, uint64_t cols, uint64_t capacity) {
 // vec_pack_ctas(n) CTAs (cta_pack.cuh): each reads all the entries for the
 // width statistics (Eq. 1) and packs its own 16 groups of 32 fields; CTA 0
 // writes the whole header.  The general path's three launches (header,
-// statistics, pack) cost more than the work here.
-constexpr uint64_t kSmallPack = 16384;
+// statistics, pack) cost more than the work here, also at 65,536 entries
+// (SMALL_FIGURES).
+constexpr uint64_t kSmallPack = 65536;
 
 template <typename T>
 __global__ void __launch_bounds__(kVecThreads) k_pack_small(const T* __restrict__ src,
@@ -430,10 +431,42 @@ __global__ void __launch_bounds__(256) k_get(const ccm_header* h, const uint32_t
   if (err && bad) atomicCAS(err, CCM_OK, CCM_E_RANGE);
 }
 
+// The same for up to kGetSmall indices by one CTA, which also writes `err`
+// (for more, a launch before k_get clears it).
+constexpr uint64_t kGetSmall = 4096;
+__global__ void __launch_bounds__(1024) k_get_small(const ccm_header* h,
+                                                    const uint32_t* __restrict__ w, uint64_t rows,
+                                                    uint64_t cols, uint64_t capacity,
+                                                    const uint64_t* __restrict__ idx,
+                                                    uint32_t count, int64_t* __restrict__ out,
+                                                    int32_t* err) {
+  const HeaderView hv = load_header(h);
+  const int st = check_header(hv, rows, cols, capacity);
+  int bad = 0;
+  if (st == CCM_OK) {
+    const uint64_t n = rows * cols;
+    for (uint32_t k = threadIdx.x; k < count; k += 1024) {
+      const uint64_t e = idx[k];
+      bad |= e >= n;
+      out[k] = e < n ? decode_field(w, e, hv.width, hv.is_signed) : 0;
+    }
+  }
+  bad = __syncthreads_or(bad);
+  if (err && threadIdx.x == 0) *err = st != CCM_OK ? st : bad ? CCM_E_RANGE : CCM_OK;
+}
+
 __global__ void k_set_i32(int32_t* p, int32_t v) { *p = v; }
 
 void run_get(const ccm_matrix& a, const uint64_t* idx, uint64_t count, int64_t* out, int32_t* err,
              cudaStream_t st) {
+  if (count && count <= kGetSmall) {
+    profile_begin(st);
+    k_get_small<<<1, 1024, 0, st>>>(a.hdr, a.words, a.rows, a.cols, a.capacity, idx,
+                                    (uint32_t)count, out, err);
+    profile_end(st);
+    note_launch();
+    return;
+  }
   if (err) {
     k_set_i32<<<1, 1, 0, st>>>(err, CCM_OK);
     note_launch();
