@@ -145,9 +145,14 @@ def _check(status: int, what: str):
         raise CCMError(status, what)
 
 
-def _stream(stream=None) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream=None) -> int:
+    """The cudaStream_t of `stream` or of the current stream of the current device (its raw
+    handle: a Stream object costs more than a kernel launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def words_for(rows: int, cols: int, width: int) -> int:
@@ -163,6 +168,23 @@ class PackedMatrix:
         dev = torch.device(device) if device is not None else torch.device("cuda")
         self.buf = torch.empty(HEADER_WORDS + self.capacity, dtype=torch.int32, device=dev)
         self._host = None  # cached host copy of the header, valid until the next write
+
+    def __getstate__(self):  # a copy gets a struct of its own (_ref)
+        return {k: v for k, v in self.__dict__.items() if k != "_struct"}
+
+    def _ref(self):
+        """A reference to this matrix's ccm_matrix for one call: the struct is kept, its fields
+        are set from the object as it is now."""
+        try:
+            m, ref = self._struct
+        except AttributeError:
+            m = Matrix()
+            ref = ctypes.byref(m)
+            self._struct = m, ref
+        p = self.buf.data_ptr()
+        m.hdr, m.words = p, p + 4 * HEADER_WORDS
+        m.capacity, m.rows, m.cols = self.capacity, self.rows, self.cols
+        return ref
 
     @property
     def device(self):
@@ -254,13 +276,12 @@ def pack_into(t: torch.Tensor, out: PackedMatrix, stream=None, ws: torch.Tensor 
     """Asynchronous SM pack of a dense CUDA tensor into a preallocated matrix
     (single pass over the dense data when a workspace applies)."""
     t, rows, cols, dt = _as_dense(t)
-    m = out.c()
     if ws is None and single_pass:
         nb = workspace_bytes(OP_PACK, rows, cols, out.capacity)
         ws = torch.empty(nb, dtype=torch.uint8, device=t.device) if nb else None
-    wsp = ctypes.c_void_p(ws.data_ptr()) if ws is not None else None
-    _check(lib().ccm_pack(ctypes.c_void_p(t.data_ptr()), dt, rows, cols, ctypes.byref(m),
-                          wsp, ws.numel() if ws is not None else 0, _stream(stream)), "ccm_pack")
+    _check(lib().ccm_pack(t.data_ptr(), dt, rows, cols, out._ref(),
+                          ws.data_ptr() if ws is not None else None,
+                          ws.numel() if ws is not None else 0, _stream(stream)), "ccm_pack")
     out._written()
     return out
 
@@ -283,9 +304,8 @@ def unpack(a: PackedMatrix, dtype=torch.int64, out: torch.Tensor | None = None, 
     if out is None:
         out = torch.empty((a.rows, a.cols), dtype=dtype, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    m = a.c()
-    _check(lib().ccm_unpack(ctypes.byref(m), ctypes.c_void_p(out.data_ptr()), dt,
-                            ctypes.c_void_p(err.data_ptr()), _stream(stream)), "ccm_unpack")
+    _check(lib().ccm_unpack(a._ref(), out.data_ptr(), dt, err.data_ptr(), _stream(stream)),
+           "ccm_unpack")
     if check:
         _check(int(err.item()), "ccm_unpack")
     return out
@@ -293,12 +313,11 @@ def unpack(a: PackedMatrix, dtype=torch.int64, out: torch.Tensor | None = None, 
 
 def get(a: PackedMatrix, idx: torch.Tensor, stream=None, check: bool = True) -> torch.Tensor:
     """Entries at flat row-major indices i*cols + j (int64 CUDA tensor)."""
-    idx = idx.to(device=a.device, dtype=torch.int64).contiguous()
+    if idx.dtype != torch.int64 or idx.device != a.device or not idx.is_contiguous():
+        idx = idx.to(device=a.device, dtype=torch.int64).contiguous()
     out = torch.empty(idx.numel(), dtype=torch.int64, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    m = a.c()
-    _check(lib().ccm_get(ctypes.byref(m), ctypes.c_void_p(idx.data_ptr()), idx.numel(),
-                         ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(err.data_ptr()),
+    _check(lib().ccm_get(a._ref(), idx.data_ptr(), idx.numel(), out.data_ptr(), err.data_ptr(),
                          _stream(stream)), "ccm_get")
     if check:
         _check(int(err.item()), "ccm_get")
@@ -332,9 +351,7 @@ def bound_matmul(a: PackedMatrix, b: PackedMatrix) -> int:
 
 
 def add_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, stream=None) -> PackedMatrix:
-    ma, mb, mc = a.c(), b.c(), c.c()
-    _check(lib().ccm_add(ctypes.byref(ma), ctypes.byref(mb), ctypes.byref(mc), None, 0,
-                         _stream(stream)), "ccm_add")
+    _check(lib().ccm_add(a._ref(), b._ref(), c._ref(), None, 0, _stream(stream)), "ccm_add")
     c._written()
     return c
 
@@ -346,9 +363,7 @@ def add(a: PackedMatrix, b: PackedMatrix, capacity: int | None = None, stream=No
 
 
 def scale_into(a: PackedMatrix, s: int, c: PackedMatrix, stream=None) -> PackedMatrix:
-    ma, mc = a.c(), c.c()
-    _check(lib().ccm_scale(ctypes.byref(ma), int(s), ctypes.byref(mc), None, 0, _stream(stream)),
-           "ccm_scale")
+    _check(lib().ccm_scale(a._ref(), int(s), c._ref(), None, 0, _stream(stream)), "ccm_scale")
     c._written()
     return c
 
@@ -382,10 +397,8 @@ def matvec_into(a: PackedMatrix, x: PackedMatrix, y: PackedMatrix, ws: torch.Ten
                 stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATVEC, a.rows, a.cols, 1, a.device)
-    ma, mx, my = a.c(), x.c(), y.c()
-    _check(lib().ccm_matvec(ctypes.byref(ma), ctypes.byref(mx), ctypes.byref(my),
-                            ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream)),
-           "ccm_matvec")
+    _check(lib().ccm_matvec(a._ref(), x._ref(), y._ref(), ws.data_ptr(), ws.numel(),
+                            _stream(stream)), "ccm_matvec")
     y._written()
     return y
 
@@ -427,10 +440,8 @@ def matmul_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, path: int = M
                 ws: torch.Tensor | None = None, stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATMUL, a.rows, a.cols, b.cols, a.device)
-    ma, mb, mc = a.c(), b.c(), c.c()
-    _check(lib().ccm_matmul(ctypes.byref(ma), ctypes.byref(mb), ctypes.byref(mc), int(path),
-                            ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream)),
-           "ccm_matmul")
+    _check(lib().ccm_matmul(a._ref(), b._ref(), c._ref(), int(path), ws.data_ptr(), ws.numel(),
+                            _stream(stream)), "ccm_matmul")
     c._written()
     return c
 
