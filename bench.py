@@ -344,7 +344,7 @@ def run_gpu(args, rank, world, local_rank):
     if rank != 0:
         return None
     hbm, peak_kind = peaks()
-    kernels = {"pack": "ge::k_pack_local<int64_t, 8>", "unpack": "ge::k_unpack_ge<int64_t, 8>",
+    kernels = {"pack": "ge::k_pack_local<int64_t, 8>", "unpack": "k_unpack_pairs<int64_t>",
                "add": "ge::k_ew_lanes<OpAdd> (+ k_ew spec/finish, which return at once)",
                "scale": "ge::k_ew_lanes<OpScale<true>> (+ k_ew spec/finish, which return at once)",
                "matvec": "mvs::k_mv<byte lanes, narrow>"}
