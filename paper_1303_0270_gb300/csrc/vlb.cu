@@ -88,13 +88,14 @@ __global__ void __launch_bounds__(1024) k_vlb_scan(uint64_t* __restrict__ block_
   const int k = 32 - __clz((int)hdr->reserved0);  // bit length of the largest L
   if (threadIdx.x == 0) s_carry = 0;
   __syncthreads();
+  // (the next step's sums are loaded before this step's scan: a step is a chain
+  // of one load and three barriers)
+  uint64_t next = threadIdx.x < nblocks ? block_off[threadIdx.x] : 0;
   for (uint64_t base = 0; base < nblocks; base += blockDim.x) {
     const uint64_t b = base + threadIdx.x;
-    uint64_t v = 0;
-    if (b < nblocks) {
-      const uint64_t cnt = umin((uint64_t)kBlock, n - b * kBlock);
-      v = block_off[b] + (uint64_t)k * cnt;
-    }
+    uint64_t v = next;
+    next = b + blockDim.x < nblocks ? block_off[b + blockDim.x] : 0;
+    if (b < nblocks) v += (uint64_t)k * umin((uint64_t)kBlock, n - b * kBlock);
     // inclusive warp scan, then across warps
     uint64_t x = v;
     for (int d = 1; d < 32; d <<= 1) {
