@@ -25,10 +25,9 @@
 //
 // Measured on GB300 (whole call; before: e4m3 digits in one-CTA tiles, or the
 // CUDA cores above 16 bits): 4096^3 at 4 / 8 / 12 / 16 signed bits 0.21 / 0.39 /
-// 0.92 / 1.31 -> 0.14 / 0.15 / 0.55 / 0.56 ms; 3001 x 2503 x 3500 at 20 x 18
-// bits 8.30 -> 0.37 ms.  What bounds it: the L2, which feeds the stages about
-// 46 bytes per clock and SM; above 32-bit sums also the conversions of short
-// runs (12 x 12 bits: runs of 256).
+// 0.92 / 1.31 -> 0.14 / 0.14 / 0.36 / 0.51 ms; 3001 x 2503 x 3500 at 20 x 18
+// bits 8.30 -> 0.33 ms.  What bounds it: the L2, which feeds the stages about
+// 46 bytes per clock and SM.
 //
 // Kernels:
 //   k_planes  packed A and B -> fp16 digit planes, K-major (B transposed)
@@ -303,9 +302,11 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
   return r;
 }
 
+// (At its default scope: what it orders are tensor-memory reads, fenced before
+// it; a release at cluster scope is a memory barrier, which made a flush of an
+// accumulator take some 4000 cycles: 4096^3 at 12 bits 431 us, now 255.)
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr)
-               : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr) : "memory");
 }
 
 __device__ __forceinline__ uint32_t ld_remote(uint32_t cluster_addr) {
