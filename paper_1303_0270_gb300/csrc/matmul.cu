@@ -212,11 +212,10 @@ int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, in
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
   if (path == CCM_MATMUL_TENSOR && (!nibble_digits(a, b) || !matmul_tc_applies(a, b)))
     return CCM_E_SHAPE;
-  bool tc = path != CCM_MATMUL_CUDACORE && matmul_tc_applies(a, b);
-  if (tc && ws_bytes < c_scratch_bytes(m, n) + matmul_tc_bytes(a, b)) {
-    if (path == CCM_MATMUL_TENSOR) return CCM_E_CAPACITY;
-    tc = false;
-  }
+  // A workspace of the least size may lack room for the planes: same words from
+  // the CUDA cores.  ccm_workspace_bytes always has the room.
+  const bool tc = path != CCM_MATMUL_CUDACORE && matmul_tc_applies(a, b) &&
+                  ws_bytes >= c_scratch_bytes(m, n) + matmul_tc_bytes(a, b);
   int64_t* cs = (int64_t*)ws;
   InitArgs ia{};
   ia.out = c.hdr;

@@ -81,3 +81,16 @@ def test_small_capacity_and_small_workspace(ccm, ba, bb):
     ws = torch.empty(need, dtype=torch.uint8, device=device())
     ccm.matmul_into(pa, pb, c, ws=ws)
     assert_same_packed(c, o, "small workspace")
+
+
+def test_tensor_path_takes_the_least_workspace(ccm):
+    """The explicit tensor path accepts every workspace that holds C and a byte
+    per field and 4-bit digit, also without room for the planes."""
+    import torch
+    m, k, n = 128, 200, 256
+    a, b = _rand(3, (m, k), 4, 1), _rand(4, (k, n), 4, 1)
+    pa, pb = ccm.pack(to_dev(a)), ccm.pack(to_dev(b))
+    ws = torch.empty(m * n * 8 + 256 + 128 * 256 + 256 * 256, dtype=torch.uint8, device=device())
+    c = ccm.PackedMatrix(m, n, ccm.words_for(m, n, 64))
+    ccm.matmul_into(pa, pb, c, path=ccm.MATMUL_TENSOR, ws=ws)
+    assert_same_packed(c, oracle.matmul(oracle.pack(a), oracle.pack(b)), "least workspace")
