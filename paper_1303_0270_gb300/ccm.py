@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import torch
 
@@ -159,6 +160,19 @@ def words_for(rows: int, cols: int, width: int) -> int:
     return int(lib().ccm_words_for(rows, cols, width))
 
 
+class _Args(threading.local):
+    """The matrix arguments of a call, kept per thread: making the structs costs more than
+    filling them (three of them 2.1 us against 1.2), and the library reads them while another
+    thread may be making a call on the same matrix."""
+
+    def __init__(self):
+        structs = [Matrix() for _ in range(3)]
+        self.slots = [(m, ctypes.byref(m)) for m in structs]
+
+
+_args = _Args()
+
+
 class PackedMatrix:
     """A matrix in SM form on the GPU: one int32 tensor = header + words."""
 
@@ -169,18 +183,10 @@ class PackedMatrix:
         self.buf = torch.empty(HEADER_WORDS + self.capacity, dtype=torch.int32, device=dev)
         self._host = None  # cached host copy of the header, valid until the next write
 
-    def __getstate__(self):  # a copy gets a struct of its own (_ref)
-        return {k: v for k, v in self.__dict__.items() if k != "_struct"}
-
-    def _ref(self):
-        """A reference to this matrix's ccm_matrix for one call: the struct is kept, its fields
-        are set from the object as it is now."""
-        try:
-            m, ref = self._struct
-        except AttributeError:
-            m = Matrix()
-            ref = ctypes.byref(m)
-            self._struct = m, ref
+    def _ref(self, slot: int):
+        """A reference to this matrix's ccm_matrix as argument `slot` of one call: a struct of the
+        calling thread, filled from the object as it is now."""
+        m, ref = _args.slots[slot]
         p = self.buf.data_ptr()
         m.hdr, m.words = p, p + 4 * HEADER_WORDS
         m.capacity, m.rows, m.cols = self.capacity, self.rows, self.cols
@@ -279,7 +285,7 @@ def pack_into(t: torch.Tensor, out: PackedMatrix, stream=None, ws: torch.Tensor 
     if ws is None and single_pass:
         nb = workspace_bytes(OP_PACK, rows, cols, out.capacity)
         ws = torch.empty(nb, dtype=torch.uint8, device=t.device) if nb else None
-    _check(lib().ccm_pack(t.data_ptr(), dt, rows, cols, out._ref(),
+    _check(lib().ccm_pack(t.data_ptr(), dt, rows, cols, out._ref(0),
                           ws.data_ptr() if ws is not None else None,
                           ws.numel() if ws is not None else 0, _stream(stream)), "ccm_pack")
     out._written()
@@ -304,7 +310,7 @@ def unpack(a: PackedMatrix, dtype=torch.int64, out: torch.Tensor | None = None, 
     if out is None:
         out = torch.empty((a.rows, a.cols), dtype=dtype, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    _check(lib().ccm_unpack(a._ref(), out.data_ptr(), dt, err.data_ptr(), _stream(stream)),
+    _check(lib().ccm_unpack(a._ref(0), out.data_ptr(), dt, err.data_ptr(), _stream(stream)),
            "ccm_unpack")
     if check:
         _check(int(err.item()), "ccm_unpack")
@@ -317,7 +323,7 @@ def get(a: PackedMatrix, idx: torch.Tensor, stream=None, check: bool = True) -> 
         idx = idx.to(device=a.device, dtype=torch.int64).contiguous()
     out = torch.empty(idx.numel(), dtype=torch.int64, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    _check(lib().ccm_get(a._ref(), idx.data_ptr(), idx.numel(), out.data_ptr(), err.data_ptr(),
+    _check(lib().ccm_get(a._ref(0), idx.data_ptr(), idx.numel(), out.data_ptr(), err.data_ptr(),
                          _stream(stream)), "ccm_get")
     if check:
         _check(int(err.item()), "ccm_get")
@@ -351,7 +357,7 @@ def bound_matmul(a: PackedMatrix, b: PackedMatrix) -> int:
 
 
 def add_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, stream=None) -> PackedMatrix:
-    _check(lib().ccm_add(a._ref(), b._ref(), c._ref(), None, 0, _stream(stream)), "ccm_add")
+    _check(lib().ccm_add(a._ref(0), b._ref(1), c._ref(2), None, 0, _stream(stream)), "ccm_add")
     c._written()
     return c
 
@@ -363,7 +369,7 @@ def add(a: PackedMatrix, b: PackedMatrix, capacity: int | None = None, stream=No
 
 
 def scale_into(a: PackedMatrix, s: int, c: PackedMatrix, stream=None) -> PackedMatrix:
-    _check(lib().ccm_scale(a._ref(), int(s), c._ref(), None, 0, _stream(stream)), "ccm_scale")
+    _check(lib().ccm_scale(a._ref(0), int(s), c._ref(1), None, 0, _stream(stream)), "ccm_scale")
     c._written()
     return c
 
@@ -397,7 +403,7 @@ def matvec_into(a: PackedMatrix, x: PackedMatrix, y: PackedMatrix, ws: torch.Ten
                 stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATVEC, a.rows, a.cols, 1, a.device)
-    _check(lib().ccm_matvec(a._ref(), x._ref(), y._ref(), ws.data_ptr(), ws.numel(),
+    _check(lib().ccm_matvec(a._ref(0), x._ref(1), y._ref(2), ws.data_ptr(), ws.numel(),
                             _stream(stream)), "ccm_matvec")
     y._written()
     return y
@@ -440,7 +446,7 @@ def matmul_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, path: int = M
                 ws: torch.Tensor | None = None, stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATMUL, a.rows, a.cols, b.cols, a.device)
-    _check(lib().ccm_matmul(a._ref(), b._ref(), c._ref(), int(path), ws.data_ptr(), ws.numel(),
+    _check(lib().ccm_matmul(a._ref(0), b._ref(1), c._ref(2), int(path), ws.data_ptr(), ws.numel(),
                             _stream(stream)), "ccm_matmul")
     c._written()
     return c
