@@ -28,6 +28,7 @@
 
 #include "async_copy.cuh"
 #include "group_engine.cuh"
+#include "host_cache.h"
 #include "pack_engine.cuh"
 
 namespace ccm {
@@ -1262,15 +1263,24 @@ inline int ew_grid(uint64_t n, int per_sm) {
   return (int)umin(umax(want, 1), (uint64_t)num_sms() * per_sm);
 }
 
-// The grid of a persistent kernel: no more CTAs than stay resident (`per_sm` is
-// kept between calls: the occupancy query is slow next to a launch).
+// CTAs of a persistent kernel that stay resident on an SM of device `dev` (kept
+// in `cache`: the occupancy query is slow next to a launch).
 template <class K>
-int resident_grid(K kernel, size_t smem, int& per_sm, uint64_t n) {
-  if (!per_sm &&
-      (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem) != cudaSuccess ||
-       per_sm < 1))
-    per_sm = 1;
-  return ew_grid(n, per_sm);
+int resident_ctas(K kernel, size_t smem, int dev, DeviceCache& cache) {
+  return cache.get(dev, 1, [&] {
+    int per_sm = 0;
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem);
+    return e == cudaSuccess ? per_sm : 0;
+  });
+}
+
+// The grid of a persistent kernel without dynamic shared memory.
+template <class K>
+int resident_grid(K kernel, DeviceCache& cache, uint64_t n) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return ew_grid(n, resident_ctas(kernel, 0, dev, cache));
 }
 
 // Launchers of one width class C, one per family of EwKind (each family is
@@ -1284,8 +1294,8 @@ int launch_ew_add(const EwCall& c, cudaStream_t st) {
   int launched = 1;
   const uint64_t n = c.rows * c.cols;
   PackedIn a{c.ha, c.wa, 0, 0, 0}, b{c.hb, c.wb, 0, 0, 0};
-  static int per_sm = 0;
-  const int g = resident_grid(k_ew<OpAdd, C, kSpec>, 0, per_sm, n);
+  static DeviceCache per_sm;
+  const int g = resident_grid(k_ew<OpAdd, C, kSpec>, per_sm, n);
   const OpAdd op{a, b};
   if (c.kind == EwKind::AddStats)
     k_ew<OpAdd, C, kStats><<<g, kThreads, 0, st>>>(op, c.out, nullptr, 0, n, 0);
@@ -1309,8 +1319,8 @@ int launch_ew_scale(const EwCall& c, cudaStream_t st) {
   int launched = 1;
   const uint64_t n = c.rows * c.cols;
   const OpScale<SMALL> op{PackedIn{c.ha, c.wa, 0, 0, 0}, c.s};
-  static int per_sm = 0;
-  const int g = resident_grid(k_ew<OpScale<SMALL>, C, kSpec>, 0, per_sm, n);
+  static DeviceCache per_sm;
+  const int g = resident_grid(k_ew<OpScale<SMALL>, C, kSpec>, per_sm, n);
   if (c.kind == EwKind::ScaleStats) {
     k_ew<OpScale<SMALL>, C, kStats><<<g, kThreads, 0, st>>>(op, c.out, nullptr, 0, n, 0);
   } else if (c.kind == EwKind::ScaleSpec) {

@@ -14,26 +14,20 @@ static void launch_lanes(const Op& op, ccm_header* out, uint32_t* words, uint64_
                          uint64_t n, int bmax, cudaStream_t st) {
   const uint32_t ww = lane_warp_words(bmax, Op::kTwoInputs ? 2 : 1, Op::kLaneGrow);
   const size_t smem = (size_t)kWarps * ww * sizeof(uint32_t);
-  static int dev_done = -1;
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev_done != dev) {
+  static DeviceCache attr;
+  attr.get(dev, 0, [&] {
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa{};
     cudaFuncGetAttributes(&fa, k_ew_lanes<Op>);  // (its static mbarriers count against optin)
-    cudaFuncSetAttribute(k_ew_lanes<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         optin - (int)fa.sharedSizeBytes);
-    dev_done = dev;
-  }
-  // (kept per width bound: the occupancy query is slow next to a launch)
-  static int per_sm_of[33] = {};
-  int& per_sm = per_sm_of[bmax < 0 || bmax > 32 ? 32 : bmax];
-  if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ew_lanes<Op>, kThreads,
-                                                                smem) != cudaSuccess ||
-                  per_sm < 1))
-    per_sm = 1;
-  const int g = ew_grid(n, per_sm);
+    return cudaFuncSetAttribute(k_ew_lanes<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin - (int)fa.sharedSizeBytes) == cudaSuccess;
+  });
+  static DeviceCache per_sm[33];  // per width bound
+  const int g = ew_grid(n, resident_ctas(k_ew_lanes<Op>, smem, dev,
+                                         per_sm[bmax < 0 || bmax > 32 ? 32 : bmax]));
   ax::launch_pdl(k_ew_lanes<Op>, dim3(g), dim3(kThreads), smem, st, op, out, words, capacity, n,
                  ww);
 }

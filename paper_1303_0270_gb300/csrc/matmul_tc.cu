@@ -45,6 +45,7 @@
 
 #include "async_copy.cuh"
 #include "ccm_device.cuh"
+#include "host_cache.h"
 #include "kernels.h"
 #include "matmul_tc.h"
 
@@ -814,15 +815,16 @@ template <int BN, bool kAcc64>
 cudaError_t launch_mm(const CUtensorMap& ta, const CUtensorMap& tb, const tc::MmArgs& args,
                       unsigned pairs, bool pdl, cudaStream_t st) {
   using G = tc::Geo<BN, kAcc64>;
-  static int dev_done = -1;  // (the attribute is the device's)
+  static DeviceCache attr;  // (the attribute is the device's)
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev_done != dev) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        tc::k_mm<BN, kAcc64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::kSmem);
-    if (e != cudaSuccess) return e;
-    dev_done = dev;
-  }
+  cudaError_t e = cudaSuccess;
+  attr.get(dev, 0, [&] {
+    e = cudaFuncSetAttribute(tc::k_mm<BN, kAcc64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)G::kSmem);
+    return e == cudaSuccess;
+  });
+  if (e != cudaSuccess) return e;
   if (pdl)
     return ax::launch_pdl(tc::k_mm<BN, kAcc64>, dim3(2 * pairs), dim3(tc::kThreads), G::kSmem, st,
                           ta, tb, args);

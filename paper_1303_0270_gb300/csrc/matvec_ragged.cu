@@ -11,6 +11,7 @@
 // before): 14 bits 392 -> 47 us (3.7 TB/s), 16 bits 335 -> 62, 32 bits 76 us
 // (5.3 TB/s).
 #include "async_copy.cuh"
+#include "host_cache.h"
 #include "kernels.h"
 #include "pack_engine.cuh"
 #include "segment_range.cuh"
@@ -114,14 +115,13 @@ void run_ragged(const ccm_matrix& a, const ccm_matrix& x, const ccm_matrix& y, v
          (uint32_t)(a.rows * nsr), DivSeg::make(nsr), (uint8_t*)ximg, yv, slot_bytes(kStageBytes, bmax),
          fresh ? 1 : 0};
   const size_t smem = (size_t)kWarps * kSlots * g.slot;
-  static int dev_done = -1;  // (the attribute is the device's)
+  static DeviceCache attr;  // (the attribute is the device's)
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev_done != dev) {
-    cudaFuncSetAttribute(k_rag, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kWarps * kSlots * (int)slot_bytes(kStageBytes, 32));
-    dev_done = dev;
-  }
+  attr.get(dev, 0, [] {  // (an error is the call's: CCM_E_CUDA)
+    return cudaFuncSetAttribute(k_rag, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kWarps * kSlots * (int)slot_bytes(kStageBytes, 32)) == cudaSuccess;
+  });
   const unsigned gi = (unsigned)umin(umax((nsr + 7) / 8, fresh ? (a.rows + 2047) / 2048 : 1),
                                      (uint64_t)num_sms() * 2);
   k_rag_init<<<gi, 256, 0, st>>>(g);

@@ -40,27 +40,25 @@ void launch_ew(int cls, const ge::EwCall& c, cudaStream_t st) {
 }  // namespace
 
 int num_sms() {
-  int dev = 0, sms = 0;
+  int dev = 0;
   cudaGetDevice(&dev);
-  static int cached_dev = -1, cached = 0;
-  if (dev != cached_dev) {
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cached = sms > 0 ? sms : 1;
-    cached_dev = dev;
-  }
-  return cached;
+  static DeviceCache sms;
+  return sms.get(dev, 1, [&] {
+    int v = 0;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v;
+  });
 }
 
 int max_smem_optin() {
-  int dev = 0, v = 0;
+  int dev = 0;
   cudaGetDevice(&dev);
-  static int cached_dev = -1, cached = 0;
-  if (dev != cached_dev) {
+  static DeviceCache bytes;
+  return bytes.get(dev, 48 * 1024, [&] {
+    int v = 0;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cached = v > 0 ? v : 48 * 1024;
-    cached_dev = dev;
-  }
-  return cached;
+    return v;
+  });
 }
 
 __global__ void k_init(InitArgs a) {
