@@ -121,8 +121,10 @@ typedef enum ccm_op {
 /* Matmul paths. */
 typedef enum ccm_matmul_path {
   CCM_MATMUL_AUTO = 0,
-  CCM_MATMUL_TENSOR = 1,  /* exact digit decomposition on the tcgen05 tensor cores (operands
-                             of at most 16 bits; AUTO takes it for wider ones too) */
+  CCM_MATMUL_TENSOR = 1,  /* exact digit decomposition on the tcgen05 tensor cores.  Asked for by
+                             name it takes operands of at most 16 bits (L = 1..4 units of 4 bits,
+                             rounded up, in the wider one) with 225 L k < 2^24 and refuses
+                             others with CCM_E_SHAPE; AUTO takes it for wider and longer ones */
   CCM_MATMUL_CUDACORE = 2 /* decode-and-multiply on the integer ALUs */
 } ccm_matmul_path;
 
@@ -239,8 +241,12 @@ ccm_status ccm_matmul(const ccm_matrix* a, const ccm_matrix* b, const ccm_matrix
 /* Device workspace needed by `op` on an m x k by k x n problem (matvec: n = 1
  * is the vector, k the inner size).  An upper bound over all operand widths
  * (for matmul: the tensor path's digit planes, three 2-byte digits per field;
- * with less, a product that would need more runs on the CUDA cores).  For
- * CCM_OP_PACK the arguments are (rows, cols, output capacity in words). */
+ * with less, down to about a quarter of a product's planes, it runs in strips
+ * of C, and below that on the CUDA cores; the least that is accepted is C in
+ * int64 and 256 bytes, for CCM_MATMUL_TENSOR and what it takes by name also L
+ * bytes per field, rows of A rounded up to 128, columns of B to 256, 128 or 64
+ * for L = 1, 2 or more, k to 128).  For CCM_OP_PACK the arguments are
+ * (rows, cols, output capacity in words). */
 size_t ccm_workspace_bytes(int op, uint64_t m, uint64_t k, uint64_t n);
 
 /* Synchronous copy of a device header to host memory (waits for `stream`). */

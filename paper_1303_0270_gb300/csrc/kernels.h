@@ -78,7 +78,7 @@ void run_repack(const ccm_matrix& in, int width, int is_signed, const ccm_matrix
 size_t matmul_workspace(const ccm_matrix& a, const ccm_matrix& b);
 // What ccm_workspace_bytes gives for a shape (the widths are unknown): enough
 // for the tensor path at its widest.  With less (but at least
-// matmul_workspace) a product may run on the CUDA cores instead.
+// matmul_workspace) a product may run in strips, or on the CUDA cores.
 size_t matmul_workspace_upper(uint64_t m, uint64_t k, uint64_t n);
 int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, int path, void* ws,
                size_t ws_bytes, cudaStream_t st);

@@ -171,10 +171,13 @@ size_t c_scratch_bytes(uint64_t m, uint64_t n) {
   return ((m * n * sizeof(int64_t)) + 255) & ~(size_t)255;
 }
 
-// Digits of 4 bits of the wider operand (by the capacities) when the explicit
-// tensor path (CCM_MATMUL_TENSOR) takes the product: at most 4, with every
-// sum of 4-bit digit products below 2^24; else 0.
-int nibble_digits(const ccm_matrix& a, const ccm_matrix& b) {
+// What the explicit tensor path (CCM_MATMUL_TENSOR) takes, and the least room
+// for planes that ccm_matmul asks for then, are part of the interface: operands
+// of at most 16 bits (by their capacities) and at most 2^24 / (225 L) columns
+// of A, with one byte per field and 4 bits of the wider operand's width.  The
+// fp16 planes need up to twice that; matmul_tc_strips fits them in.
+// L, the width in units of 4 bits; 0: the path refuses the product.
+int tensor_nibbles(const ccm_matrix& a, const ccm_matrix& b) {
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
   if (!m || !n || !k) return 0;
   const int ba = width_bound(a.capacity, m * k), bb = width_bound(b.capacity, k * n);
@@ -186,36 +189,38 @@ int nibble_digits(const ccm_matrix& a, const ccm_matrix& b) {
 
 }  // namespace
 
-// One byte per field and 4-bit digit, both operands padded to whole tiles.
-static size_t nibble_bytes(uint64_t m, uint64_t k, uint64_t n, int L) {
+// The least room for planes: L bytes per field, rows, columns and k rounded up.
+static size_t least_plane_bytes(uint64_t m, uint64_t k, uint64_t n, int L) {
   auto up = [](uint64_t v, uint64_t to) { return (v + to - 1) / to * to; };
   const uint64_t kp = up(k, 128), np = up(n, L == 1 ? 256 : L == 2 ? 128 : 64);
   return up(L * up(m, 128) * kp, 256) + up(L * np * kp, 256);
 }
 
-// The least workspace ccm_matmul accepts: C in int64, plus one byte per field
-// and 4-bit digit where the explicit tensor path applies.
+// The least workspace ccm_matmul accepts: C in int64, plus the least room for
+// planes where the explicit tensor path applies.
 size_t matmul_workspace(const ccm_matrix& a, const ccm_matrix& b) {
-  const int L = nibble_digits(a, b);
+  const int L = tensor_nibbles(a, b);
   return c_scratch_bytes(a.rows, b.cols) + 256 +
-         (L ? nibble_bytes(a.rows, a.cols, b.cols, L) : 0);
+         (L ? least_plane_bytes(a.rows, a.cols, b.cols, L) : 0);
 }
 
 size_t matmul_workspace_upper(uint64_t m, uint64_t k, uint64_t n) {
   const size_t digits = m && n && k ? umax(matmul_tc_bytes_upper(m, k, n),
-                                           nibble_bytes(m, k, n, 4)) : 0;
+                                           least_plane_bytes(m, k, n, 4)) : 0;
   return c_scratch_bytes(m, n) + digits + 256;
 }
 
 int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, int path, void* ws,
                size_t ws_bytes, cudaStream_t st) {
   const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  if (path == CCM_MATMUL_TENSOR && (!nibble_digits(a, b) || !matmul_tc_applies(a, b)))
+  if (path == CCM_MATMUL_TENSOR && (!tensor_nibbles(a, b) || !matmul_tc_applies(a, b)))
     return CCM_E_SHAPE;
-  // A workspace of the least size may lack room for the planes: same words from
-  // the CUDA cores.  ccm_workspace_bytes always has the room.
-  const bool tc = path != CCM_MATMUL_CUDACORE && matmul_tc_applies(a, b) &&
-                  ws_bytes >= c_scratch_bytes(m, n) + matmul_tc_bytes(a, b);
+  // Without room for all the planes (ccm_workspace_bytes always has it) the
+  // product goes strip by strip; with hardly any, on the CUDA cores.
+  const size_t room = ws_bytes - c_scratch_bytes(m, n);
+  Strips strips{0, 0};
+  if (path != CCM_MATMUL_CUDACORE && matmul_tc_applies(a, b)) strips = matmul_tc_strips(a, b, room);
+  const bool tc = strips.rows != 0;
   int64_t* cs = (int64_t*)ws;
   InitArgs ia{};
   ia.out = c.hdr;
@@ -236,7 +241,7 @@ int run_matmul(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, in
   launch_init(ia, st);
   if (m && n && k) {
     if (tc) {
-      int rc = run_matmul_tc(a, b, c, cs, (char*)ws + c_scratch_bytes(m, n), st);
+      int rc = run_matmul_tc(a, b, c, cs, (char*)ws + c_scratch_bytes(m, n), strips, st);
       if (rc != CCM_OK) return rc;
       if (matmul_c32(c))
         run_pack_scratch32(reinterpret_cast<const int32_t*>(cs), c, st);

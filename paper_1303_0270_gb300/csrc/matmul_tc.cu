@@ -174,7 +174,9 @@ __device__ __forceinline__ uint32_t half2_bits(int x, int y, bool small) {
 struct PlaneArgs {
   const ccm_header *out, *ha, *hb;
   const uint32_t *wa, *wb;
-  uint64_t m, k, n, kp;  // kp: k rounded up to 64 (a row of a plane)
+  uint64_t row0, col0;   // the strips begin at A's row row0 and B's column col0
+  uint64_t m, k, n, kp;  // rows of A's strip, columns of B's; kp: k rounded up to 64 (a row of a plane)
+  uint64_t ldb;          // columns of B
   __half *pa, *pb;       // [da][m][kp], [db][n][kp]
   uint32_t row_runs;     // A: warp-runs (32 groups of 8 fields) per row
   uint32_t blocks_a;     // CTAs [0, blocks_a) write A's planes, the rest B's
@@ -193,7 +195,7 @@ __device__ __forceinline__ void planes_a(const PlaneArgs& a, const Split& sp) {
     const uint64_t kk = 8 * ((it - i * a.row_runs) * 32 + lane);
     if (kk >= a.kp) continue;
     int v[8];
-    decode8<B>(a.wa, i * a.k + kk, kk < a.k ? (int)umin(8, a.k - kk) : 0, sgn, v);
+    decode8<B>(a.wa, (a.row0 + i) * a.k + kk, kk < a.k ? (int)umin(8, a.k - kk) : 0, sgn, v);
     __half* dst = a.pa + i * a.kp + kk;
     for (int l = 0; l < sp.da; ++l, dst += a.m * a.kp) {
       int d[8];
@@ -220,8 +222,9 @@ __device__ __forceinline__ void planes_b(const PlaneArgs& a, const Split& sp,
   const int g8 = 8 * (tid % 8), kpair = tid / 8, cnt = min(8, cols - g8);
   const uint64_t row = k0 + 2 * kpair;
   int v0[8], v1[8];
-  decode8<B>(a.wb, row * a.n + j0 + g8, row < a.k ? cnt : 0, sgn, v0);
-  decode8<B>(a.wb, (row + 1) * a.n + j0 + g8, row + 1 < a.k ? cnt : 0, sgn, v1);
+  const uint64_t e0 = row * a.ldb + a.col0 + j0 + g8;
+  decode8<B>(a.wb, e0, row < a.k ? cnt : 0, sgn, v0);
+  decode8<B>(a.wb, e0 + a.ldb, row + 1 < a.k ? cnt : 0, sgn, v1);
   const int col = tid / 4, q = tid % 4;
   __half* dst = a.pb + (j0 + col) * a.kp + k0 + 16 * q;
   for (int l = 0; l < sp.db; ++l, dst += a.n * a.kp) {
@@ -246,7 +249,7 @@ __device__ __forceinline__ void planes_b(const PlaneArgs& a, const Split& sp,
   M(1) M(2) M(3) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12) M(13) M(14) M(15) M(16) M(17) \
   M(18) M(19) M(20) M(21) M(22) M(23) M(24) M(25) M(26) M(27) M(28) M(29) M(30) M(31)
 
-// Both operands' planes in one launch.  The bytes are b/8 in and 2 d out per
+// The planes of a strip of A and of one of B (or of one of the two) in one launch.  The bytes are b/8 in and 2 d out per
 // field; what is left beside them is the cutting of the fields, so the widths
 // are compile-time bodies chosen from the headers.
 __global__ void __launch_bounds__(256) k_planes(const __grid_constant__ PlaneArgs a) {
@@ -387,8 +390,8 @@ __device__ __forceinline__ void tmem_fence_after() {
 struct MmArgs {
   ccm_header* out;  // C header: status, width statistics
   const ccm_header *ha, *hb;
-  void* c;          // C, m x n row-major, int64 or int32
-  uint64_t m, n;
+  void* c;          // the strip of C: m x n, rows ldc apart, int64 or int32
+  uint64_t m, n, ldc;
   uint32_t k_blocks;
   uint32_t tiles_m, tiles_n;
   int c32;          // 1: C is stored as int32 (the output capacity bounds its width by 31)
@@ -455,7 +458,8 @@ __device__ __forceinline__ void add_run(const uint32_t (&r)[16], int shift,
 // consecutive lanes: through a transposing tile, kCCols columns at a time.
 template <int BN, bool kAcc64, typename T, typename UAcc, typename Acc>
 __device__ __forceinline__ void store_tile(const UAcc (&acc)[BN / 2], Acc* st, int lane, T* c,
-                                           uint64_t row0, uint64_t col0, uint64_t m, uint64_t n) {
+                                           uint64_t row0, uint64_t col0, uint64_t m, uint64_t n,
+                                           uint64_t ldc) {
   constexpr int W = Geo<BN, kAcc64>::kCCols, kRows = 32 / W;
   const int r0 = lane / W, cl = lane % W;
   const int rows = row0 < m ? (int)umin(32, m - row0) : 0;
@@ -466,12 +470,12 @@ __device__ __forceinline__ void store_tile(const UAcc (&acc)[BN / 2], Acc* st, i
     __syncwarp();
     const uint64_t col = col0 + c0 + cl;
     if (col < n) {
-      T* dst = c + (row0 + r0) * n + col;
+      T* dst = c + (row0 + r0) * ldc + col;
       const Acc* src = st + r0 * (W + 1) + cl;
 #pragma unroll 8
       for (int r = 0; r < 32; r += kRows) {
         if (r + r0 < rows) *dst = (T)src[r * (W + 1)];
-        dst += kRows * n;
+        dst += kRows * ldc;
       }
     }
     __syncwarp();
@@ -683,11 +687,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (args.c32)
         store_tile<BN, kAcc64, int32_t>(acc, reinterpret_cast<Acc*>(cst), lane,
                                         reinterpret_cast<int32_t*>(args.c), row0, col0, args.m,
-                                        args.n);
+                                        args.n, args.ldc);
       else
         store_tile<BN, kAcc64, int64_t>(acc, reinterpret_cast<Acc*>(cst), lane,
                                         reinterpret_cast<int64_t*>(args.c), row0, col0, args.m,
-                                        args.n);
+                                        args.n, args.ldc);
     }
     const uint64_t orv64 = warp_or64((uint64_t)orv);
     const uint32_t neg = __any_sync(0xffffffffu, (Acc)sgn < 0);
@@ -799,9 +803,35 @@ bool matmul_tc_applies(const ccm_matrix& a, const ccm_matrix& b) {
   return tc::encode_fn() != nullptr;
 }
 
-size_t matmul_tc_bytes(const ccm_matrix& a, const ccm_matrix& b) {
+// All of C where the planes of both operands fit.  Else the fewest strips (then
+// the fewest plane elements written: B's are written again for every strip of
+// A) whose planes fit, in steps of 32 rows and columns.  Up to kMaxParts of each:
+// the least workspace that ccm_matmul accepts for the explicit tensor path
+// never needs more, and with less room than about a quarter of the planes the
+// CUDA cores take the product.  4096^3 in the least workspace (in brackets: with
+// room for all): 4 bits 199 us (139), 12 bits 460 (362), 16 bits 564 (507); on
+// the CUDA cores 33 to 107 times as long.
+Strips matmul_tc_strips(const ccm_matrix& a, const ccm_matrix& b, size_t room) {
+  constexpr uint64_t kMaxParts = 4;
+  const uint64_t m = a.rows, k = a.cols, n = b.cols;
   const tc::Bounds r = tc::bounds_of(a, b);
-  return tc::plane_bytes(a.rows, a.cols, b.cols, r.d.da, r.d.db);
+  if (tc::plane_bytes(m, k, n, r.d.da, r.d.db) <= room) return Strips{m, n};
+  Strips best{0, 0};
+  uint64_t best_parts = 0, best_written = 0;
+  for (uint64_t pm = 1; pm <= kMaxParts; ++pm)
+    for (uint64_t pn = 1; pn <= kMaxParts; ++pn) {
+      const Strips s{umin(m, tc::round_up((m + pm - 1) / pm, 32)),
+                     umin(n, tc::round_up((n + pn - 1) / pn, 32))};
+      if (tc::plane_bytes(s.rows, k, s.cols, r.d.da, r.d.db) > room) continue;
+      const uint64_t written = r.d.da * m + r.d.db * n * (pn > 1 ? pm : 1);
+      if (!best_parts || pm * pn < best_parts ||
+          (pm * pn == best_parts && written < best_written)) {
+        best = s;
+        best_parts = pm * pn;
+        best_written = written;
+      }
+    }
+  return best;
 }
 
 size_t matmul_tc_bytes_upper(uint64_t m, uint64_t k, uint64_t n) {
@@ -834,20 +864,34 @@ cudaError_t launch_mm(const CUtensorMap& ta, const CUtensorMap& tb, const tc::Mm
 
 }  // namespace
 
-int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, void* c_scratch,
-                  void* ws, cudaStream_t st) {
-  const uint64_t m = a.rows, k = a.cols, n = b.cols;
-  const tc::Bounds r = tc::bounds_of(a, b);
-  const uint64_t kp = tc::round_up(k, 64);
-  const bool pdl = !profile_armed();
-  __half* pa = (__half*)ws;
-  __half* pb = (__half*)((char*)ws + tc::round_up(2 * (uint64_t)r.d.da * m * kp, 256));
+namespace {
+
+// C's strip of `rows` x `cols` from row0, col0 on: the planes that are not in
+// place yet, then their product.
+struct StripCall {
+  const ccm_matrix &a, &b, &c;
+  void* c_scratch;
+  __half *pa, *pb;
+  tc::Bounds r;
+  uint64_t row0, col0, rows, cols;
+  bool planes_a, planes_b;
+  bool pdl;
+};
+
+int run_strip(const StripCall& s, cudaStream_t st) {
+  const ccm_matrix &a = s.a, &b = s.b, &c = s.c;
+  const tc::Bounds& r = s.r;
+  const uint64_t m = s.rows, k = a.cols, n = s.cols, kp = tc::round_up(k, 64);
+  const bool pdl = s.pdl;
   {
-    tc::PlaneArgs p{c.hdr, a.hdr, b.hdr, a.words, b.words, m, k, n, kp, pa, pb, 0, 0, 0};
+    tc::PlaneArgs p{c.hdr, a.hdr, b.hdr, a.words, b.words, s.row0, s.col0, m, k, n, kp, b.cols,
+                    s.pa, s.pb, 0, 0, 0};
     p.row_runs = (uint32_t)((kp / 8 + 31) / 32);
-    p.blocks_a = (uint32_t)umin((m * p.row_runs + 7) / 8, (uint64_t)num_sms() * 32);
+    p.blocks_a =
+        s.planes_a ? (uint32_t)umin((m * p.row_runs + 7) / 8, (uint64_t)num_sms() * 32) : 0;
     p.tiles_k = (uint32_t)(kp / 64);
-    const unsigned grid = (unsigned)(p.blocks_a + p.tiles_k * ((n + 63) / 64));
+    const uint64_t tiles_b = s.planes_b ? p.tiles_k * ((n + 63) / 64) : 0;
+    const unsigned grid = (unsigned)(p.blocks_a + tiles_b);
     if (pdl)
       ax::launch_pdl(tc::k_planes, dim3(grid), dim3(256), 0, st, p);
     else
@@ -876,14 +920,17 @@ int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c,
   }
   const uint32_t sub = bn > 128 ? 1 : 2;
   CUtensorMap ta, tb;
-  if (!tc::make_map(&ta, pa, kp, m, r.d.da, 128, sub) ||
-      !tc::make_map(&tb, pb, kp, n, r.d.db, (uint32_t)bn / 2, sub))
+  if (!tc::make_map(&ta, s.pa, kp, m, r.d.da, 128, sub) ||
+      !tc::make_map(&tb, s.pb, kp, n, r.d.db, (uint32_t)bn / 2, sub))
     return CCM_E_CUDA;
-  tc::MmArgs args{c.hdr, a.hdr, b.hdr, c_scratch, m, n, (uint32_t)((k + tc::kBK - 1) / tc::kBK),
-                  (uint32_t)tiles_m, (uint32_t)((n + bn - 1) / bn), matmul_c32(c) ? 1 : 0};
+  const bool c32 = matmul_c32(c);
+  const uint64_t at = s.row0 * b.cols + s.col0;
+  void* cs = c32 ? (void*)((int32_t*)s.c_scratch + at) : (void*)((int64_t*)s.c_scratch + at);
+  tc::MmArgs args{c.hdr, a.hdr, b.hdr, cs, m, n, b.cols, (uint32_t)((k + tc::kBK - 1) / tc::kBK),
+                  (uint32_t)tiles_m, (uint32_t)((n + bn - 1) / bn), c32 ? 1 : 0};
   const unsigned grid = (unsigned)umin((uint64_t)args.tiles_m * args.tiles_n, pairs);
   cudaError_t e = cudaErrorInvalidValue;
-  profile_begin(st);
+  profile_begin(st);  // (of the first strip's product; run_matmul_tc ends it)
   if (acc32) {
     switch (bn) {
       case 256: e = launch_mm<256, false>(ta, tb, args, grid, pdl, st); break;
@@ -898,9 +945,27 @@ int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c,
       default: e = launch_mm<64, true>(ta, tb, args, grid, pdl, st); break;
     }
   }
-  profile_end(st);
   note_launch();
   return e == cudaSuccess ? CCM_OK : CCM_E_CUDA;
+}
+
+}  // namespace
+
+int run_matmul_tc(const ccm_matrix& a, const ccm_matrix& b, const ccm_matrix& c, void* c_scratch,
+                  void* ws, const Strips& s, cudaStream_t st) {
+  const tc::Bounds r = tc::bounds_of(a, b);
+  const uint64_t kp = tc::round_up(a.cols, 64);
+  __half* pa = (__half*)ws;
+  __half* pb = (__half*)((char*)ws + tc::round_up(2 * (uint64_t)r.d.da * s.rows * kp, 256));
+  const bool pdl = !profile_armed();
+  int rc = CCM_OK;
+  for (uint64_t i = 0; i < a.rows && rc == CCM_OK; i += s.rows)
+    for (uint64_t j = 0; j < b.cols && rc == CCM_OK; j += s.cols)
+      rc = run_strip({a, b, c, c_scratch, pa, pb, r, i, j, umin(s.rows, a.rows - i),
+                      umin(s.cols, b.cols - j), j == 0, i == 0 || s.cols < b.cols, pdl},
+                     st);
+  profile_end(st);
+  return rc;
 }
 
 }  // namespace ccm
