@@ -37,6 +37,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCols = 8192;       // x of at most 8192 entries per matrix
 constexpr uint32_t kDefaultStageBytes = 3072;
+constexpr uint32_t kShortRow = 12;   // segments of a row from which field_range is ahead of lane_range
 
 struct Mat {
   const ccm_header* ha;
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_batch_mv(const __grid_constant_
     };
     bool ok = true;
     if (job.nseg)
-      ok = matrix_range(job.view, ring, job.seg0, job.seg0 + job.nseg, code_width(job.code),
+      ok = matrix_range<kShortRow>(job.view, ring, job.seg0, job.seg0 + job.nseg, code_width(job.code),
                         code_signed(job.code), code_mode(job.code), next);
     else
       next();

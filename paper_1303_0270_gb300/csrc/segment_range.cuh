@@ -15,7 +15,9 @@
 // and x of more than 14 bits has no byte images; they take a field per lane
 // instead: a segment is b whole words, so along a row a lane's shift is fixed
 // and its word advances by b, and each field is one 64-bit multiply-add with x
-// as int32.
+// as int32 (field_range).  On rows of a few segments a lane has a segment again,
+// every lane at another field of its own, so that neither the words nor x meet
+// in a bank (lane_range).
 //
 // Row sums.  Rows of 32 segments or more: the lanes add to a running sum of the
 // warp's current row, reduced (redux.sync on 26-bit parts) and added to y with
@@ -307,11 +309,84 @@ __device__ __forceinline__ bool field_range(const MatView& M, Ring& ring, uint32
   return true;
 }
 
+// Segments [r0, r1), a segment per lane and its fields one by one, at run-time
+// width (V as above): lane l takes the fields l, l + 1, ... of its segment, round
+// its end.  For rows of fewer than kShortRow segments (the caller's): field_range
+// sums every row over the warp, which on such rows takes longer than the
+// products.  Bound by the integer pipe (about 13 instructions per field).
+// Measured on GB300 (2,500 matrices at 12 bits, x of 16 bits, us per batch;
+// field_range / this): 2500 x 16 901 / 306, 625 x 64 304 / 154, 200 x 200 219 /
+// 154, 156 x 256 141 / 142, 125 x 320 156 / 148; 100 x 400 180 against 210 for a
+// form of this that was 7 % slower at 320.
+// A function of its own: inlined, it had k_batch_mv spill registers on the other
+// paths (2 to 4 %).  The copies of the first stages are under way when it is
+// called; it returns the ring's slot and phase, or kGaveUp.
+constexpr uint32_t kGaveUp = 0xffffffffu;
+
+// (A pointer into shared memory that comes as an argument is a generic one.)
+__device__ __forceinline__ uint32_t ld_shared(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+template <bool SHORT, bool SGN, typename V>
+__device__ __noinline__ uint32_t lane_range(MatView M, Ring ring, uint32_t r0, uint32_t r1, int b) {
+  const uint32_t lane = threadIdx.x % 32, sh = 32 - b;
+  const uint32_t nsr = M.nsr, ss = 32 * lane_segments(ring.stage_bytes, b);
+  const int* xi = reinterpret_cast<const int*>(M.ximg);
+  // fields of a segment (of the only one of a row, rounded up to a power of two:
+  // x is zero past the end)
+  const uint32_t len = !SHORT ? 32u : 1u << (32 - __clz((int)M.n - 1));
+  for (uint32_t g0 = r0; g0 < r1; g0 += ss) {
+    if (!ring.wait()) {
+      ring.drain(g0, r1, ss);
+      return kGaveUp;
+    }
+    const uint32_t words = ax::smem_u32(ring.mem + ring.slot * ring.slot_bytes);
+    const uint32_t g1 = min(g0 + ss, r1);
+    const uint32_t q0 = M.row_of(g0), s0 = g0 - q0 * nsr;
+    const uint32_t bit0 = (uint32_t)M.bit_of(q0, s0, b) & 127u;
+#pragma unroll 1
+    for (uint32_t g = g0 + lane; g < g1; g += 32) {
+      const uint32_t q = M.row_of(g), s = g - q * nsr;
+      const uint32_t bit = bit0 + ((q - q0) * M.n + 32u * s - 32u * s0) * (uint32_t)b;
+      const int* x = xi + 32 * s;
+      int64_t acc = 0;
+#pragma unroll 8
+      for (uint32_t j = 0; j < len; ++j) {
+        const uint32_t e = (j + lane) & (len - 1), at = bit + e * (uint32_t)b;
+        const uint32_t w = words + (at >> 5) * 4;
+        const uint32_t t = __funnelshift_r(ld_shared(w), ld_shared(w + 4), at) << sh;
+        const V v = SGN ? (V)((int)t >> sh) : (V)(t >> sh);
+        acc += (long long)v * __ldg(x + e);
+      }
+      add_y(M.y, q, acc);
+    }
+    ring.release(M, b, g0, r1, ss);
+  }
+  return ring.slot | ring.phase << 8;
+}
+
 // Segments [r0, r1) of a matrix of fields of b bits (1 .. 32): false when a
 // wait gave up.
-template <class F>
+template <uint32_t kShortRow, class F>
 __device__ __forceinline__ bool matrix_range(const MatView& M, Ring& ring, uint32_t r0, uint32_t r1,
                                              int b, bool sgn, XMode mode, F started) {
+  if (mode == kFields && M.nsr < kShortRow) {
+    ring.start(M, b, r0, r1, 32 * lane_segments(ring.stage_bytes, b));
+    started();
+    const uint32_t at =
+        M.n < 32 ? (sgn ? lane_range<true, true, int>(M, ring, r0, r1, b)
+                        : lane_range<true, false, long long>(M, ring, r0, r1, b))
+                 : (sgn ? lane_range<false, true, int>(M, ring, r0, r1, b)
+                        : b < 32 ? lane_range<false, false, int>(M, ring, r0, r1, b)
+                                 : lane_range<false, false, long long>(M, ring, r0, r1, b));
+    if (at == kGaveUp) return false;
+    ring.slot = at & 255u;
+    ring.phase = at >> 8;
+    return true;
+  }
   if (mode == kFields)
     return sgn ? field_range<true, int>(M, ring, r0, r1, b, started)
                : b < 32 ? field_range<false, int>(M, ring, r0, r1, b, started)
