@@ -162,9 +162,11 @@ size_t pack_workspace(uint64_t rows, uint64_t cols, uint64_t capacity) {
 // A small dense input (n <= kSmallPack entries) packed in one launch by
 // vec_pack_ctas(n) CTAs (cta_pack.cuh): each reads all the entries for the
 // width statistics (Eq. 1) and packs its own 16 groups of 32 fields; CTA 0
-// writes the whole header.  The general path's three launches (header,
-// statistics, pack) cost more than the work here, also at 65,536 entries
-// (a 256 x 256 int32 pack: 22.5 us a call with three launches, now 16.4).
+// writes the whole header.  Up to 65,536 entries the general path's three
+// launches (header, tiles, re-code) cost as much or more: 8.0 to 8.5 us per call
+// queued back to back from 20,000 entries on (20.6 past 32 bits) against 6.2
+// here, 8.3 at 65,536 int64 entries; a call that the host waits for has two
+// launches less on top.
 constexpr uint64_t kSmallPack = 65536;
 
 template <typename T>
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(kVecThreads) k_pack_small(const T* __restrict_
   const uint32_t g0 = blockIdx.x * kVecGroupsPerCta;
   uint64_t orv;
   uint32_t neg;
-  vec_stats_stage([&](uint32_t i) { return (int64_t)src[i]; }, mm, g0, sm, orv, neg);
+  vec_stats_stage(src, mm, g0, sm, orv, neg);
   const int b = width_from_stats(orv, neg);
   const uint64_t nw = words_for(mm, b), dw = data_words(mm, b);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -626,7 +628,7 @@ __global__ void __launch_bounds__(kVecThreads) k_pack_vec(ccm_header* out, uint3
   const uint32_t g0 = blockIdx.x * kVecGroupsPerCta;
   uint64_t orv;
   uint32_t neg;
-  vec_stats_stage([&](uint32_t i) { return y[i]; }, mm, g0, sm, orv, neg);
+  vec_stats_stage(y, mm, g0, sm, orv, neg);
   const int b = width_from_stats(orv, neg);
   const uint64_t nw = words_for(m, b), dw = data_words(m, b);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -643,8 +645,8 @@ __global__ void __launch_bounds__(kVecThreads) k_pack_vec(ccm_header* out, uint3
 }
 
 // Longest vector of the one-launch pack: every CTA reads all of it (512 KB at
-// this length, a few us), which up to here beats a statistics pass and a pack
-// pass (20,011 sums: 16 us).
+// this length), which up to here beats a statistics pass and a pack pass
+// (whole products of 64 columns, 65,536 rows 16.7 us, 66,000 rows 22.6).
 constexpr uint64_t kVecMax = 65536;
 
 // Pack an int64 result held in device scratch (matvec / matmul epilogue).
