@@ -37,7 +37,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCols = 8192;       // x of at most 8192 entries per matrix
 constexpr uint32_t kDefaultStageBytes = 3072;
-constexpr uint32_t kShortRow = 12;   // segments of a row from which field_range is ahead of lane_range
+constexpr uint32_t kShortRow = 8;    // segments of a row from which field_range is ahead of lane_range
 
 struct Mat {
   const ccm_header* ha;

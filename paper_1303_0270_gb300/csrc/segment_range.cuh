@@ -316,8 +316,9 @@ __device__ __forceinline__ bool field_range(const MatView& M, Ring& ring, uint32
 // products.  Bound by the integer pipe (about 13 instructions per field).
 // Measured on GB300 (2,500 matrices at 12 bits, x of 16 bits, us per batch;
 // field_range / this): 2500 x 16 901 / 306, 625 x 64 304 / 154, 200 x 200 219 /
-// 154, 156 x 256 141 / 142, 125 x 320 156 / 148; 100 x 400 180 against 210 for a
-// form of this that was 7 % slower at 320.
+// 154, 178 x 224 196 / 142.  From 8 segments on the two are even at best (156 x
+// 256 141 / 142), and with rows that end inside a word field_range is ahead
+// (3,000 of 128 x 250 140 / 145, at 4 bits 135 / 163).
 // A function of its own: inlined, it had k_batch_mv spill registers on the other
 // paths (2 to 4 %).  The copies of the first stages are under way when it is
 // called; it returns the ring's slot and phase, or kGaveUp.
