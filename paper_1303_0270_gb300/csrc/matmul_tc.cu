@@ -48,6 +48,7 @@
 #include "host_cache.h"
 #include "kernels.h"
 #include "matmul_tc.h"
+#include "matmul_tile.h"
 
 namespace ccm {
 namespace tc {
@@ -55,7 +56,6 @@ namespace tc {
 using ax::mbar_init;
 using ax::smem_u32;
 
-constexpr int kBM = 256;          // rows of C per CTA pair (128 per CTA)
 constexpr int kBK = 64;           // fp16 elements of a block of k (a 128-byte swizzled row)
 constexpr uint32_t kGroupM = 4;   // tile rows per raster group
 constexpr int kMaxDigits = 3;
@@ -898,26 +898,10 @@ int run_strip(const StripCall& s, cudaStream_t st) {
       tc::k_planes<<<grid, 256, 0, st>>>(p);
     note_launch();
   }
-  // 32-bit accumulators when no result can leave int32.  The tile width is the
-  // one with the least loading: the L2 feeds about 46 bytes per clock and SM
-  // (BN = 256: 32 KB per block of k, 90 us at 4096^3; 128: 24 KB, 111 us), so
-  // a wave of tiles costs 128 rows of A and BN / 2 of B per CTA whatever the
-  // MMAs cost.  At 4096^3: 224 columns give exactly 4 waves, 82 us.
+  // 32-bit accumulators when no result can leave int32.
   const bool acc32 = r.ba + r.bb + bitlen_host(k) <= 31;
-  const int sizes32[] = {256, 224, 192, 128, 64}, sizes64[] = {128, 64};
-  const int* sizes = acc32 ? sizes32 : sizes64;
   const uint64_t tiles_m = (m + tc::kBM - 1) / tc::kBM, pairs = (uint64_t)num_sms() / 2;
-  int bn = 0;
-  double best = 0;
-  for (int i = 0; i < (acc32 ? 5 : 2); ++i) {
-    const uint64_t tiles = tiles_m * ((n + sizes[i] - 1) / sizes[i]);
-    const uint64_t waves = (tiles + pairs - 1) / pairs;
-    const double cost = (double)waves * (256 + sizes[i]);
-    if (!bn || cost < best) {
-      bn = sizes[i];
-      best = cost;
-    }
-  }
+  const int bn = tc::tile_columns(m, n, acc32, pairs);
   const uint32_t sub = bn > 128 ? 1 : 2;
   CUtensorMap ta, tb;
   if (!tc::make_map(&ta, s.pa, kp, m, r.d.da, 128, sub) ||
