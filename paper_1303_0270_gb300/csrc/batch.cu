@@ -37,7 +37,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCols = 8192;       // x of at most 8192 entries per matrix
 constexpr uint32_t kDefaultStageBytes = 3072;
-constexpr uint32_t kShortRow = 8;    // segments of a row from which field_range is ahead of lane_range
+constexpr uint32_t kShortRow = 16;   // segments of a row from which field_range is ahead of lane_range
 
 struct Mat {
   const ccm_header* ha;
@@ -137,8 +137,8 @@ __global__ void __launch_bounds__(kInitThreads) k_batch_init(const __grid_consta
 
 // ---------------------------------------------------------------------------
 // Unit order: a counting sort of the valid entries' units by code.  Each CTA
-// counts all the entries (their codes and unit counts are a few KB) and those
-// before its own slice, so it knows where its slice's units of every code go
+// counts all the entries (4 bytes of code and one sector of the record each: 360 KB
+// from L2 for 10,000) and those before its own slice, so it knows where its slice's units of every code go
 // without waiting for another CTA; then a warp writes an entry's units.  (By
 // one CTA, with one thread per entry: 105 us for 10,000 matrices.)
 // ---------------------------------------------------------------------------

@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_rag(const __grid_constant__
   const int b = a.ha->width;
   const MatView M{a.wa, a.ximg, a.y, (uint32_t)a.n, a.nsr, a.div.m, a.div.s1, a.div.s2};
   const XMode mode = x_mode(b, a.hx->width, a.hx->is_signed, a.nsr);
-  // (without lane_range: it would win under 65 columns, 235294 x 17 45 -> 31 us at
-  // x of 16 bits, and lose from there on, 20000 x 200 16.4 -> 17.4, and the call
-  // takes 8 registers from the other paths)
+  // (without lane_range, whose call takes 8 registers from the other paths; taken
+  // field by field it gave 45 -> 31 us at 235294 x 17 and x of 16 bits, and 16.4 ->
+  // 17.4 at 20000 x 200)
   if (!matrix_range<0>(M, ring, r0, r1, b, a.ha->is_signed != 0, mode, [] {}) &&
       lane == 0)
     set_status(a.out, CCM_E_TIMEOUT);

@@ -68,8 +68,8 @@ __host__ __device__ constexpr uint64_t digit_bytes(uint32_t nsr) {
 
 enum XMode : uint32_t { kOneDigit = 0, kTwoDigits = 1, kFields = 2 };
 
-// (Rows of a few segments stay with a segment per lane at 16 and 32 bits:
-// reducing every row costs more than the bank conflicts.)
+// (Rows under 8 segments stay with byte digits at 16 and 32 bits: reducing every
+// row costs more than the bank conflicts.)
 __device__ __forceinline__ XMode x_mode(int b, int bx, int sx, uint32_t nsr) {
   if (bx > kMaxByteX || ((b == 16 || b == 32) && nsr >= 8)) return kFields;
   return (sx ? bx <= 8 : bx <= 7) ? kOneDigit : kTwoDigits;
@@ -309,19 +309,21 @@ __device__ __forceinline__ bool field_range(const MatView& M, Ring& ring, uint32
   return true;
 }
 
-// Segments [r0, r1), a segment per lane and its fields one by one, at run-time
-// width (V as above): lane l takes the fields l, l + 1, ... of its segment, round
-// its end.  For rows of fewer than kShortRow segments (the caller's): field_range
-// sums every row over the warp, which on such rows takes longer than the
-// products.  Bound by the integer pipe (about 13 instructions per field).
-// Measured on GB300 (2,500 matrices at 12 bits, x of 16 bits, us per batch;
-// field_range / this): 2500 x 16 901 / 306, 625 x 64 304 / 154, 200 x 200 219 /
-// 154, 178 x 224 196 / 142.  From 8 segments on the two are even at best (156 x
-// 256 141 / 142), and with rows that end inside a word field_range is ahead
-// (3,000 of 128 x 250 140 / 145, at 4 bits 135 / 163).
-// A function of its own: inlined, it had k_batch_mv spill registers on the other
-// paths (2 to 4 %).  The copies of the first stages are under way when it is
-// called; it returns the ring's slot and phase, or kGaveUp.
+// Segments [r0, r1), a segment per lane and its fields two by two, at run-time
+// width (V as above).  Lane l begins with pair `turn` of its segment and goes
+// round its end: where all begin at pair l, up to 11 lanes' words lie in one bank at some widths
+// (30 bits; by counting); with this turn 2.4 on average over widths and row
+// lengths, at most 3.5.  For rows of fewer
+// than kShortRow segments (the caller's): field_range sums every row over the
+// warp, which on such rows takes longer than the products.  Bound by the integer
+// pipe (about 10 instructions per field).  Measured on GB300 (2,500 matrices at
+// 12 bits, x of 16 bits, us per batch; field_range / this): 5714 x 7 2025 / 595,
+// 2500 x 16 900 / 252, 625 x 64 303 / 130, 200 x 200 218 / 139, 156 x 256 141 /
+// 126, 100 x 400 180 / 170, 83 x 480 (15 segments) 171 / 162; at 16 segments
+// field_range takes 121.  (Fields one by one, 14 instructions each: 154 at 625 x
+// 64, 154 at 200 x 200.)  A function of its own: inlined, it had k_batch_mv spill
+// registers on the other paths (2 to 4 %).  The copies of the first stages are
+// under way when it is called; it returns the ring's slot and phase, or kGaveUp.
 constexpr uint32_t kGaveUp = 0xffffffffu;
 
 // (A pointer into shared memory that comes as an argument is a generic one.)
@@ -336,9 +338,10 @@ __device__ __noinline__ uint32_t lane_range(MatView M, Ring ring, uint32_t r0, u
   const uint32_t lane = threadIdx.x % 32, sh = 32 - b;
   const uint32_t nsr = M.nsr, ss = 32 * lane_segments(ring.stage_bytes, b);
   const int* xi = reinterpret_cast<const int*>(M.ximg);
-  // fields of a segment (of the only one of a row, rounded up to a power of two:
-  // x is zero past the end)
-  const uint32_t len = !SHORT ? 32u : 1u << (32 - __clz((int)M.n - 1));
+  // pairs of a segment (of the only one of a row, rounded up to a power of two: x
+  // is zero past the end)
+  const uint32_t pairs = !SHORT ? 16u : M.n <= 2 ? 1u : 1u << (31 - __clz((int)M.n - 1));
+  const uint32_t turn = 11 * (lane + (lane >> 4));  // (lane l's first pair)
   for (uint32_t g0 = r0; g0 < r1; g0 += ss) {
     if (!ring.wait()) {
       ring.drain(g0, r1, ss);
@@ -354,13 +357,16 @@ __device__ __noinline__ uint32_t lane_range(MatView M, Ring ring, uint32_t r0, u
       const uint32_t bit = bit0 + ((q - q0) * M.n + 32u * s - 32u * s0) * (uint32_t)b;
       const int* x = xi + 32 * s;
       int64_t acc = 0;
-#pragma unroll 8
-      for (uint32_t j = 0; j < len; ++j) {
-        const uint32_t e = (j + lane) & (len - 1), at = bit + e * (uint32_t)b;
+#pragma unroll 4
+      for (uint32_t j = 0; j < pairs; ++j) {
+        const uint32_t e = 2 * ((j + turn) & (pairs - 1)), at = bit + e * (uint32_t)b;
         const uint32_t w = words + (at >> 5) * 4;
-        const uint32_t t = __funnelshift_r(ld_shared(w), ld_shared(w + 4), at) << sh;
-        const V v = SGN ? (V)((int)t >> sh) : (V)(t >> sh);
-        acc += (long long)v * __ldg(x + e);
+        const uint32_t w0 = ld_shared(w), w1 = ld_shared(w + 4), w2 = ld_shared(w + 8);
+        const uint32_t lo = __funnelshift_r(w0, w1, at), hi = __funnelshift_r(w1, w2, at);
+        const uint32_t t0 = lo << sh, t1 = __funnelshift_rc(lo, hi, b) << sh;
+        const int2 xv = __ldg(reinterpret_cast<const int2*>(x + e));
+        acc += (long long)(SGN ? (V)((int)t0 >> sh) : (V)(t0 >> sh)) * xv.x;
+        acc += (long long)(SGN ? (V)((int)t1 >> sh) : (V)(t1 >> sh)) * xv.y;
       }
       add_y(M.y, q, acc);
     }
