@@ -26,8 +26,8 @@
 // Measured on GB300 (whole call; before: e4m3 digits in one-CTA tiles, or the
 // CUDA cores above 16 bits): 4096^3 at 4 / 8 / 12 / 16 signed bits 0.21 / 0.39 /
 // 0.92 / 1.31 -> 0.14 / 0.14 / 0.36 / 0.51 ms; 3001 x 2503 x 3500 at 20 x 18
-// bits 8.30 -> 0.33 ms.  What bounds it: the L2, which feeds the stages about
-// 46 bytes per clock and SM.
+// bits 8.30 -> 0.33 ms.  What bounds it, by the times over tile widths: the L2,
+// which feeds the stages about 46 bytes per clock and SM.
 //
 // Kernels:
 //   k_planes  packed A and B -> fp16 digit planes, K-major (B transposed)

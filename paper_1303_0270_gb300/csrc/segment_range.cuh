@@ -311,12 +311,12 @@ __device__ __forceinline__ bool field_range(const MatView& M, Ring& ring, uint32
 
 // Segments [r0, r1), a segment per lane and its fields two by two, at run-time
 // width (V as above).  Lane l begins with pair `turn` of its segment and goes
-// round its end: where all begin at pair l, up to 11 lanes' words lie in one bank at some widths
-// (30 bits; by counting); with this turn 2.4 on average over widths and row
-// lengths, at most 3.5.  For rows of fewer
-// than kShortRow segments (the caller's): field_range sums every row over the
-// warp, which on such rows takes longer than the products.  Bound by the integer
-// pipe (about 10 instructions per field).  Measured on GB300 (2,500 matrices at
+// round its end: where all begin at pair l, up to 11 lanes' words lie in one bank
+// at some widths (30 bits; by counting); with this turn 2.4 on average over widths
+// and row lengths, at most 3.5.  For rows of fewer than kShortRow segments (the
+// caller's): field_range sums every row over the warp, which on such rows takes
+// longer than the products.  Bound by the integer pipe (about 10 instructions per
+// field).  Measured on GB300 (2,500 matrices at
 // 12 bits, x of 16 bits, us per batch; field_range / this): 5714 x 7 2025 / 595,
 // 2500 x 16 900 / 252, 625 x 64 303 / 130, 200 x 200 218 / 139, 156 x 256 141 /
 // 126, 100 x 400 180 / 170, 83 x 480 (15 segments) 171 / 162; at 16 segments

@@ -30,10 +30,10 @@ def _pack(ccm, v, b):
     return ccm.pack_into(to_dev(v), m)
 
 
-# (rows, columns): 1 to 9 segments a row, whole and ragged, more rows than a stage holds
-SHAPES = [(300, 1), (700, 16), (257, 31), (64, 32), (300, 33), (100, 64), (90, 97), (41, 200),
-          (33, 224), (50, 225), (37, 256), (20, 257)]
-X = [(15, 1), (15, 0), (24, 1), (31, 0)]
+# (rows, columns): 1 to 16 segments a row, whole and ragged, more rows than a stage holds
+SHAPES = [(300, 1), (300, 2), (300, 3), (700, 16), (257, 31), (64, 32), (300, 33), (100, 64),
+          (90, 97), (41, 200), (33, 224), (50, 225), (37, 256), (20, 257), (40, 480), (19, 481)]
+X = [(15, 1), (15, 0), (24, 1), (31, 0), (8, 1)]  # (8 bits: int32 too at 16 and 32 bits of A)
 
 
 def _oracle(a, x):
