@@ -10,6 +10,12 @@ ccm = pytest.importorskip("paper_1303_0270_gb300.ccm")
 serve = pytest.importorskip("paper_1303_0270_gb300.serve")
 
 
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1303_0270_gb300 import build
+    build.build()
+
+
 def _up(v, to):
     return (v + to - 1) // to * to
 
