@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 import torch
@@ -162,7 +163,7 @@ def words_for(rows: int, cols: int, width: int) -> int:
 
 class _Args(threading.local):
     """The matrix arguments of a call, kept per thread: making the structs costs more than
-    filling them (three of them 2.1 us against 1.2), and the library reads them while another
+    filling them (three of them 2.1 us against 0.75), and the library reads them while another
     thread may be making a call on the same matrix."""
 
     def __init__(self):
@@ -171,6 +172,7 @@ class _Args(threading.local):
 
 
 _args = _Args()
+_fill_matrix = struct.Struct("=2Q3q").pack_into  # the fields of Matrix in one call
 
 
 class PackedMatrix:
@@ -183,13 +185,12 @@ class PackedMatrix:
         self.buf = torch.empty(HEADER_WORDS + self.capacity, dtype=torch.int32, device=dev)
         self._host = None  # cached host copy of the header, valid until the next write
 
-    def _ref(self, slot: int):
-        """A reference to this matrix's ccm_matrix as argument `slot` of one call: a struct of the
-        calling thread, filled from the object as it is now."""
-        m, ref = _args.slots[slot]
+    def _ref(self, slot):
+        """A reference to this matrix's ccm_matrix for one call: `slot` (one of _args.slots),
+        filled from the object as it is now."""
+        m, ref = slot
         p = self.buf.data_ptr()
-        m.hdr, m.words = p, p + 4 * HEADER_WORDS
-        m.capacity, m.rows, m.cols = self.capacity, self.rows, self.cols
+        _fill_matrix(m, 0, p, p + 4 * HEADER_WORDS, self.capacity, self.rows, self.cols)
         return ref
 
     @property
@@ -285,7 +286,7 @@ def pack_into(t: torch.Tensor, out: PackedMatrix, stream=None, ws: torch.Tensor 
     if ws is None and single_pass:
         nb = workspace_bytes(OP_PACK, rows, cols, out.capacity)
         ws = torch.empty(nb, dtype=torch.uint8, device=t.device) if nb else None
-    _check(lib().ccm_pack(t.data_ptr(), dt, rows, cols, out._ref(0),
+    _check(lib().ccm_pack(t.data_ptr(), dt, rows, cols, out._ref(_args.slots[0]),
                           ws.data_ptr() if ws is not None else None,
                           ws.numel() if ws is not None else 0, _stream(stream)), "ccm_pack")
     out._written()
@@ -310,8 +311,8 @@ def unpack(a: PackedMatrix, dtype=torch.int64, out: torch.Tensor | None = None, 
     if out is None:
         out = torch.empty((a.rows, a.cols), dtype=dtype, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    _check(lib().ccm_unpack(a._ref(0), out.data_ptr(), dt, err.data_ptr(), _stream(stream)),
-           "ccm_unpack")
+    _check(lib().ccm_unpack(a._ref(_args.slots[0]), out.data_ptr(), dt, err.data_ptr(),
+                            _stream(stream)), "ccm_unpack")
     if check:
         _check(int(err.item()), "ccm_unpack")
     return out
@@ -323,8 +324,8 @@ def get(a: PackedMatrix, idx: torch.Tensor, stream=None, check: bool = True) -> 
         idx = idx.to(device=a.device, dtype=torch.int64).contiguous()
     out = torch.empty(idx.numel(), dtype=torch.int64, device=a.device)
     err = torch.empty(1, dtype=torch.int32, device=a.device)
-    _check(lib().ccm_get(a._ref(0), idx.data_ptr(), idx.numel(), out.data_ptr(), err.data_ptr(),
-                         _stream(stream)), "ccm_get")
+    _check(lib().ccm_get(a._ref(_args.slots[0]), idx.data_ptr(), idx.numel(), out.data_ptr(),
+                         err.data_ptr(), _stream(stream)), "ccm_get")
     if check:
         _check(int(err.item()), "ccm_get")
     return out
@@ -357,7 +358,8 @@ def bound_matmul(a: PackedMatrix, b: PackedMatrix) -> int:
 
 
 def add_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, stream=None) -> PackedMatrix:
-    _check(lib().ccm_add(a._ref(0), b._ref(1), c._ref(2), None, 0, _stream(stream)), "ccm_add")
+    s0, s1, s2 = _args.slots
+    _check(lib().ccm_add(a._ref(s0), b._ref(s1), c._ref(s2), None, 0, _stream(stream)), "ccm_add")
     c._written()
     return c
 
@@ -369,7 +371,8 @@ def add(a: PackedMatrix, b: PackedMatrix, capacity: int | None = None, stream=No
 
 
 def scale_into(a: PackedMatrix, s: int, c: PackedMatrix, stream=None) -> PackedMatrix:
-    _check(lib().ccm_scale(a._ref(0), int(s), c._ref(1), None, 0, _stream(stream)), "ccm_scale")
+    s0, s1, _ = _args.slots
+    _check(lib().ccm_scale(a._ref(s0), int(s), c._ref(s1), None, 0, _stream(stream)), "ccm_scale")
     c._written()
     return c
 
@@ -403,7 +406,8 @@ def matvec_into(a: PackedMatrix, x: PackedMatrix, y: PackedMatrix, ws: torch.Ten
                 stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATVEC, a.rows, a.cols, 1, a.device)
-    _check(lib().ccm_matvec(a._ref(0), x._ref(1), y._ref(2), ws.data_ptr(), ws.numel(),
+    s0, s1, s2 = _args.slots
+    _check(lib().ccm_matvec(a._ref(s0), x._ref(s1), y._ref(s2), ws.data_ptr(), ws.numel(),
                             _stream(stream)), "ccm_matvec")
     y._written()
     return y
@@ -446,8 +450,9 @@ def matmul_into(a: PackedMatrix, b: PackedMatrix, c: PackedMatrix, path: int = M
                 ws: torch.Tensor | None = None, stream=None) -> PackedMatrix:
     if ws is None:
         ws = workspace(OP_MATMUL, a.rows, a.cols, b.cols, a.device)
-    _check(lib().ccm_matmul(a._ref(0), b._ref(1), c._ref(2), int(path), ws.data_ptr(), ws.numel(),
-                            _stream(stream)), "ccm_matmul")
+    s0, s1, s2 = _args.slots
+    _check(lib().ccm_matmul(a._ref(s0), b._ref(s1), c._ref(s2), int(path), ws.data_ptr(),
+                            ws.numel(), _stream(stream)), "ccm_matmul")
     c._written()
     return c
 
